@@ -29,11 +29,20 @@ struct CurveDev {
     uint64_t tab;                         // tabulated shapes: offset of the CDF table (doubles)
 };
 
+// Per-curve constants of the float draws (lc_draw.cuh): log2(lambda) = B + L K
+// with L the logarithm (K1 below the break, K2 above it) or the table's u (K =
+// U = log2 10, B = 0), as head + tail; clamp limits moved inwards by a few
+// roundings; kc scales the error bound.
+struct DrawConst {
+    float Bh, Bl, K1h, K1l, K2h, K2l, Uh, Ul, kc, lo, hi;
+};
+
 // Per-curve constants of the ERDF inverse CDF (computed once per curve on the
 // device with the same operation sequence that every draw then reuses).
 struct ErdfConst {
     double c1, c2, e1, M1, Msum, lo, hi, umin, ub;
     int32_t a1nz, a2nz;
+    DrawConst f;
 };
 
 template <typename T> struct cplx_of;
@@ -326,20 +335,6 @@ __device__ inline double erdf_density(const CurveDev& cv, double u)
 __device__ __forceinline__ double erdf_table_step(const CurveDev& cv)
 {
     return __ddiv_rn(__dsub_rn(cv.umax, cv.umin), (double)kErdfTable);
-}
-
-// Simpson's rule on interval k: (f(u_k) + 4 f(u_k + h/2) + f(u_{k+1})) h/6,
-// u_k = umin + k h.
-__device__ inline double erdf_table_interval(const CurveDev& cv, int k)
-{
-    const double h = erdf_table_step(cv);
-    const double h6 = __ddiv_rn(h, 6.0);
-    const double u0 = __dadd_rn(cv.umin, __dmul_rn((double)k, h));
-    const double u1 = __dadd_rn(cv.umin, __dmul_rn((double)(k + 1), h));
-    const double um = __dadd_rn(u0, __dmul_rn(0.5, h));
-    double sum = __dadd_rn(erdf_density(cv, u0), __dmul_rn(4.0, erdf_density(cv, um)));
-    sum = __dadd_rn(sum, erdf_density(cv, u1));
-    return __dmul_rn(sum, h6);
 }
 
 // Inverse of the tabulated CDF F[0..kErdfTable] (F in any memory space):

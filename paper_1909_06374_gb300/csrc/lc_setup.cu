@@ -1,6 +1,9 @@
 // lc_setup.cu -- setup stage of the generator (Sec. 2.1, first two steps):
 // TK95 spectrum of the Eq. 3 PSD, its FP64 variance, the target amplitudes,
 // and the ERDF draws by inverse CDF.
+#include <algorithm>
+
+#include "lc_draw.cuh"
 #include "lc_internal.h"
 
 namespace lc {
@@ -18,19 +21,48 @@ constexpr int kSpecTile = kSpecBlock * kSpecPerThread;  // bins per block
 // with |X_j|^2 replaced by P_j (the variance the PSD implies, for PSD target
 // amplitudes).  coeffs = fixed amplitude: X_j = sqrt(P_j) e^{2 pi i U2},
 // X_{N/2} = +-sqrt(P_{N/2}) with the sign of cos(2 pi U2).
+
+// Coefficient j of a curve (c = 1/(N dt f_br), nh = N/2).  y_j = f_j / f_br =
+// j c; Eq. 3 as 1 / (e^{a_lo ln y} + e^{a_hi ln y}) (one logarithm for both
+// terms); the amplitude sqrt(P/2) sqrt(-2 ln U1) as one square root: these are
+// the FP64 operations that the FP64-rate-bound kernels spend their time on.
+__device__ __forceinline__ double2 tk_bin(const CurveDev& cv, double c, bool fixed, uint64_t j, uint64_t nh, double& P)
+{
+    const uint4 w = philox(j, cv.curve_id, 0u, cv.seed);
+    const double U1 = unit_open(w.x, w.y), U2 = unit_open(w.z, w.w);
+    const double lu = fixed ? 0.0 : log(U1);  // rad^2 = -2 lu
+    double sn, cs;
+    sincospi(2.0 * U2, &sn, &cs);
+    const double ly = log((double)j * c);
+    P = 1.0 / (exp(cv.a_lo * ly) + exp(cv.a_hi * ly));
+    if (j < nh) {
+        const double a = fixed ? sqrt(P) : sqrt(-P * lu);
+        return make_double2(a * cs, a * sn);
+    }
+    return make_double2(fixed ? (cs < 0.0 ? -sqrt(P) : sqrt(P)) : sqrt(-2.0 * P * lu) * cs, 0.0);
+}
+
+// Tree sums of the block's kSpecBlock values (fixed order), in thread 0.
+__device__ __forceinline__ void spec_block_sums(double (&red)[kSpecBlock], double (&red_p)[kSpecBlock])
+{
+    __syncthreads();
+    for (int s = kSpecBlock / 2; s > 0; s >>= 1) {
+        if (threadIdx.x < s) {
+            red[threadIdx.x] += red[threadIdx.x + s];
+            red_p[threadIdx.x] += red_p[threadIdx.x + s];
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void __launch_bounds__(kSpecBlock)
 k_tk_spectrum(const CurveDev* __restrict__ curves, const int* __restrict__ cls_curves,
-              int blocks_per_curve, double2* __restrict__ spec, double* __restrict__ partial,
-              double* __restrict__ partial_p)
+              int blocks_per_curve, double2* __restrict__ spec, double* __restrict__ partial, double* __restrict__ partial_p)
 {
     const int ci = blockIdx.x / blocks_per_curve;
     const int jb = blockIdx.x % blocks_per_curve;
     const CurveDev cv = curves[cls_curves[ci]];
     const uint64_t nh = 1ull << (cv.log2n - 1);
-    // y_j = f_j / f_br = j c; Eq. 3 as 1 / (e^{a_lo ln y} + e^{a_hi ln y}) (one
-    // logarithm for both terms); the amplitude sqrt(P/2) sqrt(-2 ln U1) as one
-    // square root: these are the FP64 operations this FP64-rate-bound kernel
-    // spends its time on
     const double c = 1.0 / ((double)(1ull << cv.log2n) * cv.dt * cv.f_br);
     const bool fixed = cv.coeffs == 1;
     double acc = 0.0, acc_p = 0.0;
@@ -40,20 +72,12 @@ k_tk_spectrum(const CurveDev* __restrict__ curves, const int* __restrict__ cls_c
         if (j > nh) continue;
         double2 X = make_double2(0.0, 0.0);
         if (j > 0) {
-            const uint4 w = philox(j, cv.curve_id, 0u, cv.seed);
-            const double U1 = unit_open(w.x, w.y), U2 = unit_open(w.z, w.w);
-            const double lu = fixed ? 0.0 : log(U1);  // rad^2 = -2 lu
-            double sn, cs;
-            sincospi(2.0 * U2, &sn, &cs);
-            const double ly = log((double)j * c);
-            const double P = 1.0 / (exp(cv.a_lo * ly) + exp(cv.a_hi * ly));
+            double P;
+            X = tk_bin(cv, c, fixed, j, nh, P);
             if (j < nh) {
-                const double a = fixed ? sqrt(P) : sqrt(-P * lu);
-                X = make_double2(a * cs, a * sn);
                 acc += 2.0 * (X.x * X.x + X.y * X.y);
                 acc_p += 2.0 * P;
             } else {
-                X = make_double2(fixed ? (cs < 0.0 ? -sqrt(P) : sqrt(P)) : sqrt(-2.0 * P * lu) * cs, 0.0);
                 acc += X.x * X.x;
                 acc_p += P;
             }
@@ -63,17 +87,62 @@ k_tk_spectrum(const CurveDev* __restrict__ curves, const int* __restrict__ cls_c
     __shared__ double red[kSpecBlock], red_p[kSpecBlock];
     red[threadIdx.x] = acc;
     red_p[threadIdx.x] = acc_p;
-    __syncthreads();
-    for (int s = kSpecBlock / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            red[threadIdx.x] += red[threadIdx.x + s];
-            red_p[threadIdx.x] += red_p[threadIdx.x + s];
-        }
-        __syncthreads();
-    }
+    spec_block_sums(red, red_p);
     if (threadIdx.x == 0) {
         partial[blockIdx.x] = red[0];
         partial_p[blockIdx.x] = red_p[0];
+    }
+}
+
+// The same coefficients for a few short curves, whose tiles would occupy few
+// SMs (an SM's FP64 rate gives 1024 bins in 46 us): one bin per thread and
+// kFewBins bins per block; the partial sums, in the order of k_tk_spectrum's,
+// by k_tk_sums.  PSD targets need the sum of P as well and take k_tk_spectrum.
+constexpr int kFewBins = 64;
+__global__ void __launch_bounds__(kFewBins) k_tk_bins(const CurveDev* __restrict__ curves,
+                                                      const int* __restrict__ cls_curves, int blocks_per_curve,
+                                                      double2* __restrict__ spec)
+{
+    const CurveDev& cv = curves[cls_curves[blockIdx.x / blocks_per_curve]];
+    const uint64_t j = (uint64_t)(blockIdx.x % blocks_per_curve) * kFewBins + threadIdx.x;
+    const uint64_t nh = 1ull << (cv.log2n - 1);
+    if (j > nh) return;
+    double2 X = make_double2(0.0, 0.0);
+    if (j > 0) {
+        double P;
+        X = tk_bin(cv, 1.0 / ((double)(1ull << cv.log2n) * cv.dt * cv.f_br), cv.coeffs == 1, j, nh, P);
+    }
+    spec[cv.offh + j] = X;
+}
+
+__global__ void __launch_bounds__(kSpecBlock) k_tk_sums(const CurveDev* __restrict__ curves,
+                                                        const int* __restrict__ cls_curves, int blocks_per_curve,
+                                                        const double2* __restrict__ spec, double* __restrict__ partial, double* __restrict__ partial_p)
+{
+    const int jb = blockIdx.x % blocks_per_curve;
+    const CurveDev& cv = curves[cls_curves[blockIdx.x / blocks_per_curve]];
+    const uint64_t nh = 1ull << (cv.log2n - 1);
+    double2 X[kSpecPerThread];
+#pragma unroll
+    for (int q = 0; q < kSpecPerThread; ++q) {
+        const uint64_t j = (uint64_t)jb * kSpecTile + (uint64_t)q * kSpecBlock + threadIdx.x;
+        X[q] = j > 0 && j <= nh ? spec[cv.offh + j] : make_double2(0.0, 0.0);
+    }
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < kSpecPerThread; ++q) {
+        const uint64_t j = (uint64_t)jb * kSpecTile + (uint64_t)q * kSpecBlock + threadIdx.x;
+        if (j > nh || j == 0) continue;
+        if (j < nh) acc += 2.0 * (X[q].x * X[q].x + X[q].y * X[q].y);
+        else acc += X[q].x * X[q].x;
+    }
+    __shared__ double red[kSpecBlock], red_p[kSpecBlock];
+    red[threadIdx.x] = acc;
+    red_p[threadIdx.x] = 0.0;
+    spec_block_sums(red, red_p);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = red[0];
+        partial_p[blockIdx.x] = 0.0;
     }
 }
 
@@ -129,16 +198,34 @@ __global__ void __launch_bounds__(256) k_amplitudes(const CurveDev* __restrict__
 __global__ void k_erdf_constants(const CurveDev* __restrict__ curves, int ncurves, ErdfConst* __restrict__ out)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < ncurves) out[c] = erdf_constants(curves[c]);
+    if (c >= ncurves) return;
+    ErdfConst k = erdf_constants(curves[c]);
+    k.f = draw_constants(k);
+    out[c] = k;
+}
+
+// Tables of the float draws, copied to shared memory by every block.
+__device__ const DrawTables g_draw_tables = make_draw_tables();
+__device__ __forceinline__ void load_draw_tables(DrawTables* t)
+{
+    for (int i = threadIdx.x; i < (int)(sizeof(DrawTables) / 4); i += blockDim.x)
+        ((uint32_t*)t)[i] = ((const uint32_t*)&g_draw_tables)[i];
+}
+
+// The FP64 sequence for the draws that the float path leaves undecided.
+__device__ __noinline__ float erdf_draw_decide(const ErdfConst& k, double U) { return (float)erdf_draw(k, U); }
+__device__ __noinline__ float erdf_draw_tab_decide(const double* F, double umin, double h, double lo, double hi,
+                                                   double U)
+{
+    return (float)erdf_draw_tab(F, umin, h, lo, hi, U);
 }
 
 // ERDF draws (Sec. 2.1 second step; inverse CDF instead of slice sampling):
 // draw k uses Philox block k/2 of stream 1, words (w0,w1) for even k and
-// (w2,w3) for odd k; lambda is computed in FP64 and rounded to T.
-template <typename T>
-__global__ void k_erdf_draws(const CurveDev* __restrict__ curves, const int* __restrict__ cls_curves,
+// (w2,w3) for odd k; lambda is computed in FP64.
+__global__ void k_erdf_draws_fp64(const CurveDev* __restrict__ curves, const int* __restrict__ cls_curves,
                              int ncurves, uint32_t log2n, const ErdfConst* __restrict__ ek,
-                             T* __restrict__ x)
+                             double* __restrict__ x)
 {
     const uint64_t half = 1ull << (log2n - 1);
     const uint64_t total = (uint64_t)ncurves * half;
@@ -153,24 +240,76 @@ __global__ void k_erdf_draws(const CurveDev* __restrict__ curves, const int* __r
         const uint4 w = philox(q, cv.curve_id, 1u, cv.seed);
         const double l0 = erdf_draw(k, unit_open(w.x, w.y));
         const double l1 = erdf_draw(k, unit_open(w.z, w.w));
-        x[cv.off + 2 * q] = (T)l0;
-        x[cv.off + 2 * q + 1] = (T)l1;
+        x[cv.off + 2 * q] = l0;
+        x[cv.off + 2 * q + 1] = l1;
     }
 }
 
-// CDF tables of the tabulated ERDF shapes, one block per curve: the
-// intervals in parallel, then their sum in order by one thread.
+// The same draws rounded to float (lc_draw.cuh): a block inverts `pairs`
+// consecutive Philox blocks of one curve.  Bound by the FP64 pipe still (5 to 9
+// operations per draw, ~120 before) and by issue: 255 curves of 2^16 samples
+// 5.11 -> 0.65 ms, the 1.9e8 draws of a ragged batch 57.9 -> 7.2 ms.
+__global__ void __launch_bounds__(256) k_erdf_draws(const CurveDev* __restrict__ curves,
+                                                    const int* __restrict__ cls_curves, int chunks, uint32_t pairs,
+                                                    const ErdfConst* __restrict__ ek, float* __restrict__ x)
+{
+    __shared__ DrawTables t;
+    __shared__ ErdfConst k;
+    load_draw_tables(&t);
+    const int c = cls_curves[blockIdx.x / chunks];
+    const CurveDev& cv = curves[c];
+    if (cv.kind != 0) return;  // tabulated shapes: k_erdf_draws_tab
+    for (int i = threadIdx.x; i < (int)(sizeof(ErdfConst) / 4); i += blockDim.x)
+        ((uint32_t*)&k)[i] = ((const uint32_t*)(ek + c))[i];
+    const uint64_t cid = cv.curve_id, seed = cv.seed;
+    const uint32_t q0 = (uint32_t)(blockIdx.x % chunks) * pairs;
+    float2* __restrict__ out = (float2*)(x + cv.off);
+    __syncthreads();
+    const DrawConst d = k.f;
+    for (uint32_t q = q0 + threadIdx.x; q < q0 + pairs; q += blockDim.x) {
+        const uint4 w = philox(q, cid, 1u, seed);
+        const double U0 = unit_open_fast(w.x, w.y), U1 = unit_open_fast(w.z, w.w);
+        float l0, l1;
+        const bool ok0 = erdf_draw_fast(t, k, d, U0, l0);
+        const bool ok1 = erdf_draw_fast(t, k, d, U1, l1);
+        if (!ok0) l0 = erdf_draw_decide(k, U0);
+        if (!ok1) l1 = erdf_draw_decide(k, U1);
+        out[q] = make_float2(l0, l1);
+    }
+}
+
+// CDF tables of the tabulated ERDF shapes, one block per curve: Simpson's rule
+// on every interval, (f(u_k) + 4 f(u_k + h/2) + f(u_{k+1})) h/6 with u_k = umin
+// + k h, in parallel, then their sum in order by one thread.  Bound by the FP64
+// rate: 2 densities per interval instead of 3 (766 curves, 1.55 -> 1.13 ms).
 __global__ void __launch_bounds__(256) k_erdf_table(const CurveDev* __restrict__ curves,
                                                     const int* __restrict__ tab_curves, double* __restrict__ tab)
 {
     __shared__ double I[kErdfTable];
     const CurveDev& cv = curves[tab_curves[blockIdx.x]];
-    for (int k = threadIdx.x; k < kErdfTable; k += blockDim.x) I[k] = erdf_table_interval(cv, k);
+    {
+        // a thread's intervals are consecutive, so an interval's right end
+        // point is the next one's left (the same u, hence the same density)
+        constexpr int kPer = kErdfTable / 256;
+        const double h = erdf_table_step(cv);
+        const double h6 = __ddiv_rn(h, 6.0);
+        const int k0 = threadIdx.x * kPer;
+        double u0 = __dadd_rn(cv.umin, __dmul_rn((double)k0, h)), f0 = erdf_density(cv, u0);
+        for (int k = k0; k < k0 + kPer; ++k) {
+            const double u1 = __dadd_rn(cv.umin, __dmul_rn((double)(k + 1), h)), f1 = erdf_density(cv, u1);
+            double sum = __dadd_rn(f0, __dmul_rn(4.0, erdf_density(cv, __dadd_rn(u0, __dmul_rn(0.5, h)))));
+            sum = __dadd_rn(sum, f1);
+            I[k] = __dmul_rn(sum, h6);
+            u0 = u1;
+            f0 = f1;
+        }
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         double* F = tab + cv.tab;
         double acc = 0.0;
         F[0] = 0.0;
+#pragma unroll 8
         for (int k = 0; k < kErdfTable; ++k) {
             acc = __dadd_rn(acc, I[k]);
             F[k + 1] = acc;
@@ -180,7 +319,8 @@ __global__ void __launch_bounds__(256) k_erdf_table(const CurveDev* __restrict__
 
 // Draws of the tabulated shapes: a block stages its curve's table in shared
 // memory and inverts `pairs` Philox blocks (same stream and word use as
-// k_erdf_draws).
+// k_erdf_draws); float draws by lc_draw.cuh (766 curves of 2^16 samples 5.57
+// -> 1.98 ms).
 template <typename T>
 __global__ void __launch_bounds__(256) k_erdf_draws_tab(const CurveDev* __restrict__ curves,
                                                         const int* __restrict__ tab_cls_curves, int chunks,
@@ -188,19 +328,31 @@ __global__ void __launch_bounds__(256) k_erdf_draws_tab(const CurveDev* __restri
                                                         const double* __restrict__ tab, T* __restrict__ x)
 {
     __shared__ double F[kErdfTable + 1];
+    __shared__ DrawTables t;
     const int c = tab_cls_curves[blockIdx.x / chunks];
     const uint64_t q0 = (uint64_t)(blockIdx.x % chunks) * pairs;
     const CurveDev& cv = curves[c];
     for (int i = threadIdx.x; i <= kErdfTable; i += blockDim.x) F[i] = tab[cv.tab + i];
+    if (sizeof(T) == 4) load_draw_tables(&t);
     __syncthreads();
-    const ErdfConst k = ek[c];
+    const double klo = ek[c].lo, khi = ek[c].hi, umin = cv.umin;
+    const DrawConst d = ek[c].f;
     const double h = erdf_table_step(cv);
     for (uint64_t q = q0 + threadIdx.x; q < q0 + pairs; q += blockDim.x) {
         const uint4 w = philox(q, cv.curve_id, 1u, cv.seed);
-        const double l0 = erdf_draw_tab(F, cv.umin, h, k.lo, k.hi, unit_open(w.x, w.y));
-        const double l1 = erdf_draw_tab(F, cv.umin, h, k.lo, k.hi, unit_open(w.z, w.w));
-        x[cv.off + 2 * q] = (T)l0;
-        x[cv.off + 2 * q + 1] = (T)l1;
+        const double U0 = unit_open_fast(w.x, w.y), U1 = unit_open_fast(w.z, w.w);
+        T l0, l1;
+        if constexpr (sizeof(T) == 4) {
+            const bool ok0 = erdf_draw_tab_fast(t, F, umin, h, d, U0, l0);
+            const bool ok1 = erdf_draw_tab_fast(t, F, umin, h, d, U1, l1);
+            if (!ok0) l0 = erdf_draw_tab_decide(F, umin, h, klo, khi, U0);
+            if (!ok1) l1 = erdf_draw_tab_decide(F, umin, h, klo, khi, U1);
+        } else {
+            l0 = erdf_draw_tab(F, umin, h, klo, khi, U0);
+            l1 = erdf_draw_tab(F, umin, h, klo, khi, U1);
+        }
+        x[cv.off + 2 * q] = l0;
+        x[cv.off + 2 * q + 1] = l1;
     }
 }
 
@@ -220,14 +372,24 @@ int spec_blocks_per_curve(uint32_t log2n)
     return (int)((nh1 + kSpecTile - 1) / kSpecTile);
 }
 
-void launch_tk_spectrum(const Plan& p, const ClassInfo& k, cudaStream_t st)
+int launch_tk_spectrum(const Plan& p, const ClassInfo& k, cudaStream_t st)
 {
     const int bpc = spec_blocks_per_curve(k.log2n);
     double* part = p.d_partial + k.partial_off;
     double* part_p = p.d_partial + p.partial_total + k.partial_off;
-    k_tk_spectrum<<<k.ncurves * bpc, kSpecBlock, 0, st>>>(p.d_curves, k.d_curves, bpc, p.d_spec, part, part_p);
+    // fewer tiles than two per SM: spread over the GPU bin by bin
+    bool few = (int64_t)k.ncurves * bpc < 152 * 2;
+    for (int i = 0; few && i < k.ncurves; ++i) few = p.h_curves[k.h_curves[i]].targets == 0;
+    if (few) {
+        const int bb = (int)(((1ull << (k.log2n - 1)) + kFewBins) / kFewBins);
+        k_tk_bins<<<k.ncurves * bb, kFewBins, 0, st>>>(p.d_curves, k.d_curves, bb, p.d_spec);
+        k_tk_sums<<<k.ncurves * bpc, kSpecBlock, 0, st>>>(p.d_curves, k.d_curves, bpc, p.d_spec, part, part_p);
+    } else {
+        k_tk_spectrum<<<k.ncurves * bpc, kSpecBlock, 0, st>>>(p.d_curves, k.d_curves, bpc, p.d_spec, part, part_p);
+    }
     k_sigma<<<(k.ncurves + 127) / 128, 128, 0, st>>>(k.d_curves, k.ncurves, bpc, part, part_p, p.d_sigma,
                                                      p.d_sigma + p.ncurves);
+    return few ? 3 : 2;
 }
 
 template <typename T>
@@ -254,13 +416,25 @@ void launch_erdf_draws(const Plan& p, const ClassInfo& k, cudaStream_t st)
 {
     if (k.ntab < k.ncurves) {
         const uint64_t work = (uint64_t)k.ncurves << (k.log2n - 1);
-        k_erdf_draws<T><<<grid_for(work, 256), 256, 0, st>>>(p.d_curves, k.d_curves, k.ncurves, k.log2n,
-                                                             p.d_erdf, (T*)p.d_x);
+        if constexpr (sizeof(T) == 8) {
+            k_erdf_draws_fp64<<<grid_for(work, 256), 256, 0, st>>>(p.d_curves, k.d_curves, k.ncurves, k.log2n,
+                                                                   p.d_erdf, (double*)p.d_x);
+        } else {
+            // eight Philox blocks per thread, fewer while the grid would not fill the GPU
+            const uint64_t half = 1ull << (k.log2n - 1);
+            uint64_t pairs = std::min<uint64_t>(half, 2048);
+            while (pairs > 256 && work / pairs < 152 * 8) pairs /= 2;
+            const int chunks = (int)(half / pairs);
+            k_erdf_draws<<<k.ncurves * chunks, 256, 0, st>>>(p.d_curves, k.d_curves, chunks, (uint32_t)pairs,
+                                                             p.d_erdf, (float*)p.d_x);
+        }
     }
     if (k.ntab) {
-        // up to 8192 Philox blocks (16384 draws) per block of threads
+        // up to 8192 Philox blocks (16384 draws) per block of threads, fewer
+        // while the grid would not fill the GPU
         const uint64_t half = 1ull << (k.log2n - 1);
-        const uint64_t pairs = half < 8192 ? half : 8192;
+        uint64_t pairs = half < 8192 ? half : 8192;
+        while (pairs > 512 && (half / pairs) * k.ntab < 152 * 4) pairs /= 2;
         const int chunks = (int)(half / pairs);
         k_erdf_draws_tab<T><<<k.ntab * chunks, 256, 0, st>>>(p.d_curves, k.d_tab_curves, chunks, pairs, p.d_erdf,
                                                              p.d_tab, (T*)p.d_x);
