@@ -91,4 +91,92 @@ __device__ __forceinline__ void dft_regs(cplx<T> (&u)[R])
     }
 }
 
+// ---------------------------------------------------- fixed float rounding
+// The iteration ranks what the transforms return, so a float transform has to
+// round the same way in every kernel that computes it, however the compiler
+// would contract its products.  These forms write every rounding down; the
+// products that FMA leaves unrounded are the ones of the kernels' plain
+// expressions as nvcc contracts them.  FP64 transforms run one kernel per
+// length and take the plain expressions.
+
+// a b with one product of each component rounded first: a.y b.y of the real
+// part, and of the imaginary part a.y b.x (cmul_a) or a.x b.y (cmul_b).
+__device__ __forceinline__ float2 cmul_a(float2 a, float2 b)
+{
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ float2 cmul_b(float2 a, float2 b)
+{
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ double2 cmul_a(double2 a, double2 b) { return cmul(a, b); }
+__device__ __forceinline__ double2 cmul_b(double2 a, double2 b) { return cmul(a, b); }
+
+// a +- b as one packed operation (two float roundings, one issue slot): the
+// three transform kernels of an iteration of 4096 x 2^16 samples 1.754 -> 1.735
+// ms, of one 2^17 curve 15.9 -> 15.2 us.
+__device__ __forceinline__ unsigned long long pack2(float2 a)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ float2 add_fixed(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 sub_fixed(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+
+// rot16 with every rounding written down.
+template <bool INV>
+__device__ __forceinline__ float2 rot16_fixed(float2 b, int t)
+{
+    if (t == 0) return b;
+    if (t == 4) return INV ? make_float2(-b.y, b.x) : make_float2(b.y, -b.x);
+    const float c = (float)cos16(t);
+    const float s = INV ? (float)cos16(t + 12) : -(float)cos16(t + 12);
+    const bool x1 = t == 6 && !INV, y1 = t != 2;
+    return make_float2(x1 ? __fmaf_rn(-b.y, s, __fmul_rn(b.x, c)) : __fmaf_rn(b.x, c, -__fmul_rn(b.y, s)),
+                       y1 ? __fmaf_rn(b.y, c, __fmul_rn(b.x, s)) : __fmaf_rn(b.x, s, __fmul_rn(b.y, c)));
+}
+
+// dft_regs with every rounding written down.
+template <typename T, int R, bool INV>
+__device__ __forceinline__ void dft_fixed(cplx<T> (&u)[R])
+{
+    if constexpr (sizeof(T) == 8) {
+        dft_regs<T, R, INV>(u);
+    } else {
+        constexpr int LR = ilog2c(R);
+        BitrevSwaps<0, R, float2>::run(u);
+#pragma unroll
+        for (int s = 1; s <= LR; ++s) {
+            const int m = 1 << s, h = m >> 1;
+#pragma unroll
+            for (int g = 0; g < R; g += m) {
+#pragma unroll
+                for (int j = 0; j < h; ++j) {
+                    const float2 a = u[g + j];
+                    const float2 b = rot16_fixed<INV>(u[g + j + h], j * (16 / m));
+                    u[g + j] = add_fixed(a, b);
+                    u[g + j + h] = sub_fixed(a, b);
+                }
+            }
+        }
+    }
+}
+
 }  // namespace lc

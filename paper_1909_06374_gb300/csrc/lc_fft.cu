@@ -38,7 +38,7 @@ struct SmemTw {
     bool three;
     __device__ __forceinline__ cplx<T> operator()(uint32_t e) const
     {
-        cplx<T> w = cmul(t1[(e >> 9) & (kTwLevel - 1)], t0[e & (kTwLevel - 1)]);
+        cplx<T> w = cmul_b(t1[(e >> 9) & (kTwLevel - 1)], t0[e & (kTwLevel - 1)]);
         if (three) w = cmul(t2[e >> 18], w);
         return w;
     }
@@ -77,6 +77,39 @@ __device__ __forceinline__ SmemTw<T> build_smem_tw(cplx<T>* mem, const cplx<T>* 
     }
     __syncthreads();
     return tw;
+}
+
+// The same twiddles for the few-column tiles: W^e as the same product of the
+// same entries, read straight from the class table (a block has too few
+// elements to pay for the shared levels), and only W_R^e in shared memory.  For
+// M <= 2^18 (two levels).
+template <typename T>
+struct DirectTw {
+    const cplx<T>* rt;
+    const cplx<T>* tR;
+    uint64_t M;
+    __device__ __forceinline__ cplx<T> operator()(uint32_t e) const
+    {
+        return cmul_b(twiddle_M<T>(rt, (uint64_t)(e & ~0x1ffu), M), twiddle_M<T>(rt, (uint64_t)(e & 0x1ffu), M));
+    }
+};
+template <typename T>
+__device__ __forceinline__ DirectTw<T> build_direct_tw(cplx<T>* mem, const cplx<T>* __restrict__ rt, int log2M, int LR)
+{
+    DirectTw<T> tw;
+    tw.rt = rt;
+    tw.tR = mem;
+    tw.M = 1ull << log2M;
+    for (int x = threadIdx.x; x < (1 << LR); x += blockDim.x)
+        mem[x] = twiddle_M<T>(rt, (uint64_t)x << (log2M - LR), tw.M);
+    __syncthreads();
+    return tw;
+}
+template <bool SMALL, typename T>
+__device__ __forceinline__ auto build_tw(cplx<T>* mem, const cplx<T>* __restrict__ rt, int log2M, int LR)
+{
+    if constexpr (SMALL) return build_direct_tw<T>(mem, rt, log2M, LR);
+    else return build_smem_tw<T>(mem, rt, log2M, LR);
 }
 
 // Table e^{-2 pi i k/N}, k < N/2, computed in FP64 and rounded once to T.
@@ -167,14 +200,18 @@ __global__ void __launch_bounds__(256) k_fft_pass(const PassArgs a)
 // (rows padded to C+1 elements; each sub-pass reads its butterflies into
 // registers, then overwrites the buffer), and stores y[(i-k)R + k + q p]
 // (coalesced along i, or along q when p = 1).
-// (FP64 keeps C = 16: with its radices a span 1 < p < C would occur.)
+// (FP64: 16, the unit its launches are counted in; it runs kSmallCols of them
+// per block, see launch_tile_lr.)
 __host__ __device__ constexpr int tile_cols(int LR, int elem_bytes)
 {
     return (LR >= 8 || elem_bytes > 8) ? 16 : (4096 >> LR);
 }
 
-template <typename T, int Q, bool INV, int LR, int C>
-__device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2p2, const SmemTw<T>& tw, int log2M)
+constexpr int kSmallCols = 4;
+constexpr int kSmallThreads = 128;
+
+template <typename T, int Q, bool INV, int LR, int C, int TH>
+__device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2p2, const cplx<T>* __restrict__ tR)
 {
     using V = cplx<T>;
     constexpr int LQ = ilog2c(Q);
@@ -183,13 +220,13 @@ __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2
     constexpr int R = 1 << LR;
     constexpr int nbq = R >> LQ;                 // butterflies per column
     constexpr int NB = nbq * C;                  // butterflies of the tile
-    constexpr int BPT = (NB + 255) / 256;        // per thread
+    constexpr int BPT = (NB + TH - 1) / TH;      // per thread
     const int p2 = 1 << log2p2;
     V u[BPT][Q];
 #pragma unroll
     for (int bi = 0; bi < BPT; ++bi) {
-        const int b = threadIdx.x + bi * 256;
-        if (NB % 256 == 0 || b < NB) {
+        const int b = threadIdx.x + bi * TH;
+        if (NB % TH == 0 || b < NB) {
             const int j = b & (C - 1), i2 = b >> LC;
 #pragma unroll
             for (int q = 0; q < Q; ++q) u[bi][q] = buf[(i2 + q * nbq) * S + j];
@@ -198,8 +235,8 @@ __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2
     __syncthreads();
 #pragma unroll
     for (int bi = 0; bi < BPT; ++bi) {
-        const int b = threadIdx.x + bi * 256;
-        if (NB % 256 == 0 || b < NB) {
+        const int b = threadIdx.x + bi * TH;
+        if (NB % TH == 0 || b < NB) {
             const int j = b & (C - 1), i2 = b >> LC;
             const int k2 = i2 & (p2 - 1);
             if (p2 > 1) {
@@ -207,12 +244,11 @@ __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2
                 const int sh = LR - LQ - log2p2;
 #pragma unroll
                 for (int q = 1; q < Q; ++q) {
-                    V w = tw.tR[(q * k2) << sh];
-                    if (INV) w.y = -w.y;
-                    u[bi][q] = cmul(u[bi][q], w);
+                    const V w = tR[(q * k2) << sh];
+                    u[bi][q] = INV ? cmul_b(u[bi][q], cconj(w)) : cmul_a(u[bi][q], w);
                 }
             }
-            dft_regs<T, Q, INV>(u[bi]);
+            dft_fixed<T, Q, INV>(u[bi]);
             const int jo = ((i2 - k2) << LQ) + k2;
 #pragma unroll
             for (int q = 0; q < Q; ++q) buf[(jo + q * p2) * S + j] = u[bi][q];
@@ -223,31 +259,38 @@ __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2
 // All radix-2^LR sub-passes of one tile of C columns, in place in `buf`: a
 // radix-2/4/8 sub-pass for LR mod 4, then radix-16 ones.  Ends with a block
 // barrier.
-template <typename T, bool INV, int LR, int C>
-__device__ __forceinline__ void tile_dft(cplx<T>* __restrict__ buf, const SmemTw<T>& tw, int log2M)
+template <typename T, bool INV, int LR, int C, int TH>
+__device__ __forceinline__ void tile_dft(cplx<T>* __restrict__ buf, const cplx<T>* __restrict__ tR)
 {
-    constexpr int rem = LR & 3;
+    // FP64 tiles of few columns: radix-4 sub-passes, four times the threads at
+    // work (a warp's FP64 operation holds its scheduler's FP64 unit for 64
+    // clocks, so few warps with long butterflies leave most of it idle)
+    constexpr int LQ = sizeof(T) == 8 && C == kSmallCols ? 2 : 4;
+    constexpr int rem = LR % LQ;
     int log2p2 = 0;
     if (rem) {
-        tile_subpass<T, (1 << (rem ? rem : 1)), INV, LR, C>(buf, 0, tw, log2M);
+        tile_subpass<T, (1 << (rem ? rem : 1)), INV, LR, C, TH>(buf, 0, tR);
         __syncthreads();
         log2p2 = rem;
     }
-    for (; log2p2 < LR; log2p2 += 4) {
-        tile_subpass<T, 16, INV, LR, C>(buf, log2p2, tw, log2M);
+    for (; log2p2 < LR; log2p2 += LQ) {
+        tile_subpass<T, (1 << LQ), INV, LR, C, TH>(buf, log2p2, tR);
         __syncthreads();
     }
 }
 
-template <typename T, int LR, bool INV, bool MULTI>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
+// SMALL: tiles of kSmallCols columns on kSmallThreads threads, for transforms
+// whose full tiles would leave most of the GPU idle (launch_tile_set).
+template <typename T, int LR, bool INV, bool MULTI, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? kSmallThreads : 256, SMALL ? 4 : (sizeof(T) == 4 && LR < 9) ? 4 : 2)
     k_fft_tile(const __grid_constant__ LaunchSet<PassArgs> set)
 {
     uint32_t blk;
     const PassArgs& a = set.pick<MULTI>(blk);
     using V = cplx<T>;
     constexpr int R = 1 << LR;
-    constexpr int C = tile_cols(LR, (int)sizeof(V));
+    constexpr int C = SMALL ? kSmallCols : tile_cols(LR, (int)sizeof(V));
+    constexpr int TH = SMALL ? kSmallThreads : 256;
     constexpr int LC = ilog2c(C);
     constexpr int S = C + 1;
     extern __shared__ __align__(16) unsigned char tile_smem[];
@@ -267,34 +310,34 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
     const uint32_t nb = 1u << log2nb;
     const uint32_t p = 1u << a.log2p;
     const uint32_t i0 = (uint32_t)ti * C;
-    constexpr int PER = R * C / 256;  // elements per thread
+    constexpr int PER = R * C / TH;  // elements per thread
     V v[PER];
 #pragma unroll
     for (int e = 0; e < PER; ++e) {  // every load in flight before any use
-        const int idx = threadIdx.x + e * 256;
+        const int idx = threadIdx.x + e * TH;
         v[e] = src[i0 + (uint32_t)(idx & (C - 1)) + (uint32_t)(idx >> LC) * nb];
     }
-    const SmemTw<T> tw = build_smem_tw<T>(twm, rt, (int)a.log2M, LR);
+    const auto tw = build_tw<SMALL, T>(twm, rt, (int)a.log2M, LR);
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
-        const int idx = threadIdx.x + e * 256;
+        const int idx = threadIdx.x + e * TH;
         const int r = idx >> LC, j = idx & (C - 1);
         V x = v[e];
         if (p > 1) {
             const uint32_t k = (i0 + (uint32_t)j) & (p - 1);
             V w = tw(((uint32_t)r * k) << (a.log2M - LR - a.log2p));
             if (INV) w.y = -w.y;
-            x = cmul(x, w);
+            x = cmul_b(x, w);
         }
         b0[r * S + j] = x;
     }
     __syncthreads();
-    tile_dft<T, INV, LR, C>(b0, tw, (int)a.log2M);
+    tile_dft<T, INV, LR, C, TH>(b0, tw.tR);
     const V* in = b0;
     const uint32_t smask = (1u << a.smp_shift) - 1u, shalf = (smask + 1u) >> 1;
     float* const smp = INV && a.smp ? a.smp + (size_t)ci * a.smp_words : nullptr;
     if (p >= (uint32_t)C) {
-        for (int idx = threadIdx.x; idx < R * C; idx += 256) {
+        for (int idx = threadIdx.x; idx < R * C; idx += TH) {
             const int q = idx >> LC, j = idx & (C - 1);
             const uint32_t i = i0 + (uint32_t)j, k = i & (p - 1);
             const uint32_t d = ((i - k) << LR) + k + (uint32_t)q * p;
@@ -303,7 +346,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
             if (smp && (d & smask) == shalf) smp[d >> a.smp_shift] = (float)y.x;
         }
     } else {  // p == 1 (the host guarantees p == 1 or p >= C): column i owns y[i R .. i R + R)
-        for (int idx = threadIdx.x; idx < R * C; idx += 256) {
+        for (int idx = threadIdx.x; idx < R * C; idx += TH) {
             const int j = idx >> LR, q = idx & (R - 1);
             const uint32_t d = ((i0 + (uint32_t)j) << LR) + (uint32_t)q;
             const V y = in[q * S + j];
@@ -446,6 +489,17 @@ __global__ void __launch_bounds__(256) k_spectral_tk(const SpecArgs a)
     }
 }
 
+// keep_phase and pack_pair of the tile path, every float rounding written down
+// (lc_dft.cuh).
+__device__ __forceinline__ float2 keep_phase_fixed(float2 X, float A)
+{
+    const float m2 = __fmaf_rn(X.x, X.x, __fmul_rn(X.y, X.y));
+    if (m2 == 0.0f) return make_float2(A, 0.0f);
+    const float s = __fmul_rn(A, rsqrtf(m2));
+    return make_float2(__fmul_rn(X.x, s), __fmul_rn(X.y, s));
+}
+__device__ __forceinline__ double2 keep_phase_fixed(double2 X, double A) { return keep_phase(X, A); }
+
 // One conjugate pair (t, M - t) of the spectral step on values held by the
 // caller: za = Z_t, zb = Z_{M-t} in, Z'_t, Z'_{M-t} out.  The arithmetic runs
 // on the representative k = min(t, M - t), as in k_spectral_iter.
@@ -460,11 +514,14 @@ __device__ __forceinline__ void spectral_pair_vals(cplx<T>& za, cplx<T>& zb, uin
     const V zk = low ? za : zb, zm = low ? zb : za;
     V E; E.x = (T)0.5 * (zk.x + zm.x); E.y = (T)0.5 * (zk.y - zm.y);
     V O; O.x = (T)0.5 * (zk.y + zm.y); O.y = (T)-0.5 * (zk.x - zm.x);
-    const V WO = cmul(W, O);
-    const V Yk = keep_phase(cadd(E, WO), Ak);
-    const V Ym = keep_phase(cconj(csub(E, WO)), Am);
+    const V WO = cmul_a(W, O);
+    const V Yk = keep_phase_fixed(cadd(E, WO), Ak);
+    const V Ym = keep_phase_fixed(cconj(csub(E, WO)), Am);
+    const V Ep = cadd(Yk, cconj(Ym));
+    const V Op = cmul_b(csub(Yk, cconj(Ym)), cconj(W));
     V Zk, Zm;
-    pack_pair(Yk, Ym, W, Zk, Zm);
+    Zk.x = Ep.x - Op.y; Zk.y = Ep.y + Op.x;
+    Zm.x = Ep.x + Op.y; Zm.y = -Ep.y + Op.x;
     za = low ? Zk : Zm;
     zb = low ? Zm : Zk;
 }
@@ -487,15 +544,16 @@ __device__ __forceinline__ void spectral_pair_tk(cplx<T>& za, cplx<T>& zb, uint3
 // and their H partner columns -- column pairs (0, p/2), then (g, p - g) -- so
 // all three steps stay in shared memory, saving two passes over the spectrum
 // and the spectral kernel.  Output: y[i R + q] for the block's columns i.
-template <typename T, int LR, bool MULTI>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
+template <typename T, int LR, bool MULTI, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? kSmallThreads : 256, SMALL ? 4 : (sizeof(T) == 4 && LR < 9) ? 4 : 2)
     k_fft_spectral(const __grid_constant__ LaunchSet<PassArgs> set, const void* __restrict__ A_all)
 {
     uint32_t blk;
     const PassArgs& a = set.pick<MULTI>(blk);
     using V = cplx<T>;
     constexpr int R = 1 << LR;
-    constexpr int C = tile_cols(LR, (int)sizeof(V));
+    constexpr int C = SMALL ? kSmallCols : tile_cols(LR, (int)sizeof(V));
+    constexpr int TH = SMALL ? kSmallThreads : 256;
     constexpr int LC = ilog2c(C);
     constexpr int S = C + 1;
     constexpr int H = C / 2;
@@ -523,36 +581,36 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
         if (j < H) return g;
         return g == 0 ? p / 2 : p - g;
     };
-    constexpr int PER = R * C / 256;  // elements per thread
+    constexpr int PER = R * C / TH;  // elements per thread
     V v[PER];
 #pragma unroll
     for (int e = 0; e < PER; ++e) {  // every load in flight before any use
-        const int idx = threadIdx.x + e * 256;
+        const int idx = threadIdx.x + e * TH;
         v[e] = src[column(idx & (C - 1)) + (uint32_t)(idx >> LC) * p];
     }
-    const SmemTw<T> tw = build_smem_tw<T>(twm, rt, (int)a.log2M, LR);
+    const auto tw = build_tw<SMALL, T>(twm, rt, (int)a.log2M, LR);
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
-        const int idx = threadIdx.x + e * 256;
+        const int idx = threadIdx.x + e * TH;
         const int r = idx >> LC, j = idx & (C - 1);
         // forward last pass: W_{R p}^{r k} = W_M^{r i} (k = i < p)
-        b0[r * S + j] = cmul(v[e], tw((uint32_t)r * column(j)));
+        b0[r * S + j] = cmul_a(v[e], tw((uint32_t)r * column(j)));
     }
     __syncthreads();
-    tile_dft<T, false, LR, C>(b0, tw, (int)a.log2M);
+    tile_dft<T, false, LR, C, TH>(b0, tw.tR);
     V* in = b0;
     // spectral step on the conjugate pairs, in place: in[q][j] = Z_{column(j) + q p}.
     // FP32: the twiddles and amplitudes of all of the thread's pairs are loaded
     // first, so that their latencies overlap (one wait instead of one per pair).
     constexpr bool kPre = sizeof(T) == 4;
-    constexpr int NP = kPre ? (R * H + 255) / 256 : 1;
+    constexpr int NP = kPre ? (R * H + TH - 1) / TH : 1;
     V Wp[NP];
     T Akp[NP], Amp[NP];
     if (kPre) {
 #pragma unroll
         for (int m = 0; m < NP; ++m) {
-            const int idx = threadIdx.x + m * 256;
-            if ((R * H) % 256 == 0 || idx < R * H) {
+            const int idx = threadIdx.x + m * TH;
+            if ((R * H) % TH == 0 || idx < R * H) {
                 const uint32_t t = column(idx & (H - 1)) + (uint32_t)(idx >> LH) * p;
                 const uint32_t k = 2 * t < M ? t : M - t;
                 Wp[m] = rt[k];
@@ -563,7 +621,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
     }
 #pragma unroll
     for (int m = 0; m < (kPre ? NP : 1); ++m)
-    for (int idx = threadIdx.x + m * 256; idx < R * H; idx += (kPre ? R * H : 256)) {
+    for (int idx = threadIdx.x + m * TH; idx < R * H; idx += (kPre ? R * H : TH)) {
         const int q = idx >> LH, j = idx & (H - 1);
         const uint32_t col = column(j);
         const uint32_t t = col + (uint32_t)q * p;
@@ -576,7 +634,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
                 V o; o.x = Y0 + YM; o.y = Y0 - YM;
                 in[0] = o;
             } else if (q == R / 2) {  // k = M/2 pairs with itself: X = conj(Z), packed 2 conj(Y)
-                const V Yh = keep_phase(cconj(in[q * S]), A[M >> 1]);
+                const V Yh = keep_phase_fixed(cconj(in[q * S]), A[M >> 1]);
                 V oh; oh.x = (T)2 * Yh.x; oh.y = -(T)2 * Yh.y;
                 in[q * S] = oh;
             } else if (q < R / 2) {
@@ -593,8 +651,8 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LR < 9) ? 4 : 2)
     }
     __syncthreads();
     // inverse first pass (span 1: no input twiddle)
-    tile_dft<T, true, LR, C>(b0, tw, (int)a.log2M);
-    for (int idx = threadIdx.x; idx < R * C; idx += 256) {
+    tile_dft<T, true, LR, C, TH>(b0, tw.tR);
+    for (int idx = threadIdx.x; idx < R * C; idx += TH) {
         const int j = idx >> LR, q = idx & (R - 1);
         dst[(column(j) << LR) + q] = in[q * S + j];
     }
@@ -685,8 +743,9 @@ bool tile_schedule_ok(uint32_t log2M, bool fp64)
 // of radix 2^LR on a length-2^log2M transform: the tile (R rows of C + 1
 // elements) and the twiddle tables.  Grows with log2M.
 template <typename T>
-static size_t tile_smem_bytes(int LR, int log2M)
+static size_t tile_smem_bytes(int LR, int log2M, bool small = false)
 {
+    if (small) return ((size_t)(kSmallCols + 1) + 1) * ((size_t)1 << LR) * sizeof(cplx<T>);
     return (((size_t)1 << LR) * (tile_cols(LR, (int)sizeof(cplx<T>)) + 1) + smem_tw_entries(log2M, LR)) *
            sizeof(cplx<T>);
 }
@@ -694,15 +753,17 @@ static size_t tile_smem_bytes(int LR, int log2M)
 // The longest transform of the tile path: M = 2^26 (N = 2^27).
 constexpr int kTileMaxLog2M = 26;
 
-template <typename T, int LR, bool MULTI>
+template <typename T, int LR, bool MULTI, bool SMALL>
 static cudaError_t tile_attrs_m(int smem)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_fft_tile<T, LR, false, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem);
+    cudaError_t e = cudaFuncSetAttribute(k_fft_tile<T, LR, false, MULTI, SMALL>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_tile<T, LR, true, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(k_fft_tile<T, LR, true, MULTI, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_spectral<T, LR, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(k_fft_spectral<T, LR, MULTI, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 smem);
     return e;
 }
 
@@ -710,8 +771,13 @@ template <typename T, int LR>
 static cudaError_t tile_attrs()
 {
     const int smem = (int)tile_smem_bytes<T>(LR, kTileMaxLog2M);
-    cudaError_t e = tile_attrs_m<T, LR, false>(smem);
-    if (e == cudaSuccess) e = tile_attrs_m<T, LR, true>(smem);
+    const int small = (int)tile_smem_bytes<T>(LR, kTileMaxLog2M, true);
+    cudaError_t e = tile_attrs_m<T, LR, false, true>(small);
+    if (e == cudaSuccess) e = tile_attrs_m<T, LR, true, true>(small);
+    if constexpr (sizeof(T) == 4) {
+        if (e == cudaSuccess) e = tile_attrs_m<T, LR, false, false>(smem);
+        if (e == cudaSuccess) e = tile_attrs_m<T, LR, true, false>(smem);
+    }
     return e;
 }
 
@@ -735,13 +801,61 @@ cudaError_t fft_kernel_attributes()
     return e;
 }
 
+// Whether a launch of `blocks` full tiles takes tiles of kSmallCols columns
+// instead: where the full tiles (four or two resident per SM) give fewer than
+// two blocks per SM, the time is one block's, and a block of a quarter of the
+// columns or less is done sooner: one 2^17 curve's three transform kernels 20.5
+// -> 14.9 us per iteration.  FP64 transforms, bound by the FP64 rate, always
+// take them, with radix-4 sub-passes: one FP64 2^14 curve 78 -> 30 us per
+// iteration, and a curve's rounding does not depend on its batch; float tiles
+// round alike in both sizes.
+static bool small_tiles(const LaunchSet<PassArgs>& s, uint32_t blocks)
+{
+    if (blocks >= 152 * 2) return false;
+    for (int i = 0; i < s.n; ++i)
+        if (s.c[i].log2M > 18) return false;  // the full tiles' twiddles have a third level there
+    return true;
+}
+
+// The launch set with every entry's blocks times f (full tiles to small ones).
+static LaunchSet<PassArgs> scaled_set(const LaunchSet<PassArgs>& s, uint32_t f)
+{
+    LaunchSet<PassArgs> r = s;
+    for (int i = 0; i < s.n; ++i) r.start[i] *= f;
+    return r;
+}
+
 // One tile pass of radix 2^LR over the launch set's classes; dynamic shared
 // memory for the longest of them.
 template <typename T, int LR, bool INV>
 static void launch_tile_lr(const LaunchSet<PassArgs>& s, uint32_t blocks, size_t smem, bool multi, cudaStream_t st)
 {
-    if (multi) k_fft_tile<T, LR, INV, true><<<blocks, 256, smem, st>>>(s);
-    else k_fft_tile<T, LR, INV, false><<<blocks, 256, smem, st>>>(s);
+    if (sizeof(T) == 8 || small_tiles(s, blocks)) {
+        constexpr uint32_t f = tile_cols(LR, (int)sizeof(cplx<T>)) / kSmallCols;
+        const LaunchSet<PassArgs> r = scaled_set(s, f);
+        smem = tile_smem_bytes<T>(LR, 0, true);
+        if (multi) k_fft_tile<T, LR, INV, true, true><<<blocks * f, kSmallThreads, smem, st>>>(r);
+        else k_fft_tile<T, LR, INV, false, true><<<blocks * f, kSmallThreads, smem, st>>>(r);
+    } else if constexpr (sizeof(T) == 4) {
+        if (multi) k_fft_tile<T, LR, INV, true, false><<<blocks, 256, smem, st>>>(s);
+        else k_fft_tile<T, LR, INV, false, false><<<blocks, 256, smem, st>>>(s);
+    }
+}
+
+template <typename T, int LR>
+static void launch_spectral_lr(const LaunchSet<PassArgs>& s, uint32_t blocks, size_t smem, bool multi, const void* A,
+                               cudaStream_t st)
+{
+    if (sizeof(T) == 8 || small_tiles(s, blocks)) {
+        constexpr uint32_t f = tile_cols(LR, (int)sizeof(cplx<T>)) / kSmallCols;
+        const LaunchSet<PassArgs> r = scaled_set(s, f);
+        smem = tile_smem_bytes<T>(LR, 0, true);
+        if (multi) k_fft_spectral<T, LR, true, true><<<blocks * f, kSmallThreads, smem, st>>>(r, A);
+        else k_fft_spectral<T, LR, false, true><<<blocks * f, kSmallThreads, smem, st>>>(r, A);
+    } else if constexpr (sizeof(T) == 4) {
+        if (multi) k_fft_spectral<T, LR, true, false><<<blocks, 256, smem, st>>>(s, A);
+        else k_fft_spectral<T, LR, false, false><<<blocks, 256, smem, st>>>(s, A);
+    }
 }
 
 template <typename T, bool INV>
@@ -778,23 +892,13 @@ static void launch_spectral_set(int LR, const LaunchSet<PassArgs>& s, uint32_t b
     size_t smem = 0;
     for (int i = 0; i < s.n; ++i) smem = std::max(smem, tile_smem_bytes<T>(LR, (int)s.c[i].log2M));
     switch (LR) {
-#define LC_FUSED_CASE(L)                                                               \
-    case L:                                                                            \
-        if (multi) k_fft_spectral<T, L, true><<<blocks, 256, smem, st>>>(s, A);         \
-        else k_fft_spectral<T, L, false><<<blocks, 256, smem, st>>>(s, A);              \
-        break;
-        LC_FUSED_CASE(5)
-        LC_FUSED_CASE(6)
-        LC_FUSED_CASE(7)
-        LC_FUSED_CASE(8)
-#undef LC_FUSED_CASE
+    case 5: launch_spectral_lr<T, 5>(s, blocks, smem, multi, A, st); break;
+    case 6: launch_spectral_lr<T, 6>(s, blocks, smem, multi, A, st); break;
+    case 7: launch_spectral_lr<T, 7>(s, blocks, smem, multi, A, st); break;
+    case 8: launch_spectral_lr<T, 8>(s, blocks, smem, multi, A, st); break;
     default:
-        if (sizeof(T) == 4 && LR == 9) {
-            if (multi) k_fft_spectral<float, 9, true><<<blocks, 256, smem, st>>>(s, A);
-            else k_fft_spectral<float, 9, false><<<blocks, 256, smem, st>>>(s, A);
-        } else {
-            set_error("internal: unsupported fused radix");
-        }
+        if (sizeof(T) == 4 && LR == 9) launch_spectral_lr<float, 9>(s, blocks, smem, multi, A, st);
+        else set_error("internal: unsupported fused radix");
         break;
     }
 }
@@ -983,7 +1087,7 @@ void launch_fft_iteration(const Plan& p, const std::vector<const ClassInfo*>& ks
             ClassState& x = cs[i];
             if (r > x.P - 2) continue;
             x.a.in = x.cur; x.a.out = x.nxt; x.a.log2p = x.log2p;
-            if (r == 0 && x.k->bucket && sizeof(T) == 4) {  // the sample sort's sample of x_adj
+            if (r == 0 && x.k->bucket) {  // the sample sort's sample of x_adj
                 x.a.smp = bucket_sample_area(*x.k);
                 x.a.smp_words = (uint32_t)bucket_curve_words(x.k->log2n);
                 x.a.smp_shift = bucket_sample_shift(x.k->log2n);
