@@ -446,7 +446,7 @@ static lc_status run_setup(Plan& p, void* out_tk, cudaStream_t st, uint64_t* lau
     p.timed_iter = false;
     launch_eff_iters(p, 0, st);
     ++*launches;
-    for (auto& k : p.classes) { launch_tk_spectrum(p, k, st); *launches += 2; }
+    for (auto& k : p.classes) *launches += (uint64_t)launch_tk_spectrum(p, k, st);
     for (auto& k : p.classes) { launch_amplitudes<T>(p, k, st); ++*launches; }
     if (out_tk) {
         for (auto& k : p.classes) {

@@ -193,7 +193,8 @@ constexpr size_t kMaxLags = 4096;
 
 // setup stage (lc_setup.cu)
 int spec_blocks_per_curve(uint32_t log2n);
-void launch_tk_spectrum(const Plan& p, const ClassInfo& k, cudaStream_t st);
+// returns the number of launches
+int launch_tk_spectrum(const Plan& p, const ClassInfo& k, cudaStream_t st);
 template <typename T> void launch_amplitudes(const Plan& p, const ClassInfo& k, cudaStream_t st);
 void launch_erdf_constants(const Plan& p, cudaStream_t st);
 // CDF tables of every curve with a tabulated ERDF shape (before the draws)
