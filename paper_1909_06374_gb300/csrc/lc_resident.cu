@@ -7,11 +7,13 @@
 //      twiddles from two small shared tables (W^t = W^{128 a} W^b);
 //   2. unpack to X_0..X_M, keep the phases, impose A, pack for the inverse;
 //   3. inverse complex FFT -> x_adj;
-//   4. stable LSD radix sort of the order keys of x_adj (4 passes of 8 bits;
+//   4. the stable rank of every x_adj (one CTA: rank_replace, by counting;
+//      clusters: LSD radix sort of the order keys, 4 passes of 8 bits with
 //      ballot-based warp multisplit, per-warp digit counts, block-wide scan);
 //   5. x[position] = s[rank].
-// A and s stream from L2.  Single CTA: the state never leaves shared memory
-// until the end of the launch.  Cluster: the length-M transform is split
+// A streams from L2, and so does s where shared memory has no room for it.
+// Single CTA: the state never leaves shared memory until the end of the
+// launch.  Cluster: the length-M transform is split
 // M = C x Mc (a cross-CTA radix-C step and local length-Mc transforms, CTA c
 // holding Z[C k + c]); the cross-CTA data goes through L2 -- on this GPU L2
 // moves ~10 TB/s between the SMs of a cluster against ~1-2.5 TB/s for
@@ -23,6 +25,7 @@
 
 #include "lc_dft.cuh"
 #include "lc_internal.h"
+#include "lc_rank.cuh"
 
 namespace lc {
 
@@ -34,7 +37,7 @@ constexpr int kResThreads = 512;
 constexpr int kResWarps = kResThreads / 32;
 constexpr uint32_t kResMinLog2 = 10;
 constexpr uint32_t kResMaxLog2 = 14;          // one CTA
-constexpr uint32_t kResAutoMaxLog2 = 12;      // the auto mode's crossover (autotune.py sweep)
+constexpr uint32_t kResAutoMaxLog2 = 12;      // the auto mode's last fused length (resident_supported)
 constexpr uint32_t kResClusterMaxLog2 = 16;   // clusters of 2 or 4 CTAs
 constexpr int kTwLo = 128;                    // low twiddle table (W^b, b < 128)
 constexpr int kTwHiMax = 64;                  // high table (W^{128 a}), Mc <= 8192
@@ -243,15 +246,13 @@ __device__ __forceinline__ double cta_sum(float v, double* red)
 // One stable LSD radix pass over the L = 2^LOG2L keys of the CTA (warp w
 // owns elements [w L/16, (w+1) L/16), lane-striped).  FIRST: keys are the
 // order keys of the x_adj floats in xa (swizzled); positions are implicit.
-// GATHER: instead of the sorted pairs, writes xn[position] = s[rank].
 // Ranking runs in two phases: the digits and ballot masks of all the warp's
 // slots (independent, so their ballot chains overlap), then the short chain
 // of per-warp digit counters in shared memory.
-template <int LOG2L, bool FIRST, bool GATHER>
+template <int LOG2L, bool FIRST>
 __device__ __forceinline__ void radix_pass(const float* __restrict__ xa, const uint32_t* __restrict__ kin,
                                            uint32_t* __restrict__ kout, const uint16_t* __restrict__ iin,
-                                           uint16_t* __restrict__ iout, float* __restrict__ xn,
-                                           const float* __restrict__ s, int shift, uint32_t* wh,
+                                           uint16_t* __restrict__ iout, int shift, uint32_t* wh,
                                            uint32_t* dbase, uint32_t* wsum)
 {
     constexpr int EW = 1 << (LOG2L - 4);  // elements per warp
@@ -307,13 +308,8 @@ __device__ __forceinline__ void radix_pass(const float* __restrict__ xa, const u
         const uint32_t d = (key >> shift) & 255u;
         const uint32_t r = (e & 1) ? (rk[e >> 1] >> 16) : (rk[e >> 1] & 0xffffu);
         const uint32_t dest = dbase[d] + wh[w * 256 + d] + r;
-        const uint32_t idx = FIRST ? (uint32_t)el : (uint32_t)iin[el];
-        if (GATHER) {
-            xn[fsw((int)idx)] = __ldg(s + dest);
-        } else {
-            kout[dest] = key;
-            iout[dest] = (uint16_t)idx;
-        }
+        kout[dest] = key;
+        iout[dest] = FIRST ? (uint16_t)el : iin[el];
     }
     __syncthreads();
     for (int q = threadIdx.x; q < kResWarps * 256; q += kResThreads) wh[q] = 0;
@@ -321,22 +317,85 @@ __device__ __forceinline__ void radix_pass(const float* __restrict__ xa, const u
 }
 
 // ------------------------------------------------------------- one CTA
-template <int LOG2L, bool CONV>
-__global__ void __launch_bounds__(kResThreads, 1) k_resident_cta(const ResArgs a)
+// Threads per CTA: 512 (the convergence test sums a thread's samples in float,
+// so there they are part of its result).  Shared memory (bytes): two
+// transform buffers (the idle one holds the ranking's counters or, up to 2^13,
+// where four bins per value still fit 16 bits, all of it), then the ranking's
+// other parts, s up to 2^12 (read from L2 above), twiddles.
+constexpr int kCtaBpv = 4;
+template <int LOG2L>
+struct CtaShape {
+    static constexpr int L = 1 << LOG2L;
+    using R = RankShape<float, LOG2L, kResThreads, kCtaBpv>;
+    static constexpr bool SHARED_S = LOG2L <= 12;
+    static constexpr size_t WST = (size_t)8 * L;
+    static constexpr size_t SLOT = WST + R::WST;
+    static constexpr size_t S = SLOT + R::SLOT;
+    static constexpr size_t SEG = S + (SHARED_S ? (size_t)4 * L : 0);
+    static constexpr size_t SPL = SEG + R::SEG;
+    static constexpr size_t TW = SPL + R::SPL;
+    static constexpr size_t BYTES = TW + kTwBytes;
+    static_assert(R::CNT <= (size_t)4 * L, "the counters fit the idle transform buffer");
+    static constexpr int MINB = LOG2L <= 12 ? 2 : 1;
+};
+
+// x[position] = s[rank] of the L values in xf (swizzled); idle: the other
+// transform buffer; both: the two of them.  Ends with a block barrier.
+template <int LOG2L>
+__device__ __forceinline__ void rank_replace(float* xf, float2* idle, unsigned char* smem, const float* s,
+                                             uint32_t* wsum, bool& warm)
 {
+    using CS = CtaShape<LOG2L>;
+    constexpr int TH = kResThreads, PER = CS::R::PER;
+    const int tid = threadIdx.x;
+    float v[PER];
+    uint32_t rk[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) v[j] = xf[fsw(tid + j * TH)];
+    RankMem<float> m;
+    m.mem = (uint32_t*)xf;
+    m.cnt = (uint32_t*)idle;
+    m.wst = (uint16_t*)(smem + CS::WST);
+    m.slot = (uint16_t*)(smem + CS::SLOT);
+    m.seg = (float2*)(smem + CS::SEG);
+    m.spl = (float*)(smem + CS::SPL);
+    m.wsum = wsum;
+    warm = cta_rank<float, LOG2L, TH, kCtaBpv, false>(m, warm, [&](int j) { return v[j]; },
+                                               [&](int i) { return xf[fsw(i)]; }, rk);
+    if (warm) {
+#pragma unroll
+        for (int j = 0; j < PER; ++j) xf[fsw(tid + j * TH)] = s[rk[j]];
+    } else {  // crowded: sorted whole, by (order key, position)
+        unsigned long long* both = (unsigned long long*)smem;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            both[tid + j * TH] = ((unsigned long long)order_key(v[j]) << 32) | (uint32_t)(tid + j * TH);
+        __syncthreads();
+        cta_bitonic<TH>(both, CS::L);
+#pragma unroll
+        for (int j = 0; j < PER; ++j) rk[j] = (uint32_t)both[tid + j * TH];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < PER; ++j) xf[fsw((int)rk[j])] = s[tid + j * TH];
+    }
+    __syncthreads();
+}
+
+template <int LOG2L, bool CONV>
+__global__ void __launch_bounds__(kResThreads, CtaShape<LOG2L>::MINB) k_resident_cta(const ResArgs a)
+{
+    using CS = CtaShape<LOG2L>;
+    constexpr int TH = kResThreads;
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int log2L = LOG2L;
-    const int L = 1 << log2L;
-    const int M = L >> 1;
+    constexpr int L = 1 << log2L;
+    constexpr int M = L >> 1;
     float2* buf0 = (float2*)smem;
     float2* buf1 = (float2*)(smem + (size_t)4 * L);
-    uint16_t* ia = (uint16_t*)(smem + (size_t)8 * L);
-    uint16_t* ib = (uint16_t*)(smem + (size_t)10 * L);
-    uint32_t* wh = (uint32_t*)(smem + (size_t)12 * L);
-    float2* twlo = (float2*)(smem + (size_t)12 * L + kWhBytes);
+    float2* twlo = (float2*)(smem + CS::TW);
     float2* twhi = twlo + kTwLo;
-    __shared__ uint32_t dbase[256];
-    __shared__ uint32_t wsum[8];
+    __shared__ uint32_t wsum[kResWarps];
     __shared__ double red[kResWarps];
 
     const int c = a.cls_curves[blockIdx.x];
@@ -349,14 +408,19 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident_cta(const ResArgs a
     const float* s = a.s + cv.off;
     float* xg = a.x + cv.off;
 
-    for (int q = threadIdx.x; q < kResWarps * 256; q += kResThreads) wh[q] = 0;
     build_tw(twlo, twhi, a.tw, log2L - 1, 1, M);
     const float2* xg2 = (const float2*)xg;
-    for (int m = threadIdx.x; m < M; m += kResThreads) buf0[swz(m)] = xg2[m];
+    for (int m = threadIdx.x; m < M; m += TH) buf0[swz(m)] = xg2[m];
+    if (CS::SHARED_S) {
+        float* ss = (float*)(smem + CS::S);
+        for (int m = threadIdx.x; m < L; m += TH) ss[m] = s[m];
+        s = ss;
+    }
     __syncthreads();
 
     float2* z = buf0;
     float2* o = buf1;
+    bool warm = false;
     for (int it = 0; it < n_act; ++it) {
         float2* Z = smem_fft<false>(z, o, log2L - 1, twlo, twhi);
         float2* Zs = (Z == buf0) ? buf1 : buf0;
@@ -364,36 +428,29 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident_cta(const ResArgs a
         __syncthreads();
         float2* X = smem_fft<true>(Zs, Z, log2L - 1, twlo, twhi);
         float2* other = (X == buf0) ? buf1 : buf0;
-        uint32_t* kX = (uint32_t*)X;
-        uint32_t* kO = (uint32_t*)other;
-        // pass 0: x_adj (in X) -> keys in other; 1: other -> X; 2: X -> other; 3: other -> x in X
-        radix_pass<LOG2L, true, false>((const float*)X, nullptr, kO, nullptr, ia, nullptr, s, 0, wh, dbase, wsum);
-        radix_pass<LOG2L, false, false>(nullptr, kO, kX, ia, ib, nullptr, s, 8, wh, dbase, wsum);
-        radix_pass<LOG2L, false, false>(nullptr, kX, kO, ib, ia, nullptr, s, 16, wh, dbase, wsum);
-        radix_pass<LOG2L, false, true>(nullptr, kO, nullptr, ia, nullptr, (float*)X, s, 24, wh, dbase, wsum);
+        rank_replace<LOG2L>((float*)X, other, smem, s, wsum, warm);
         z = X;
         o = other;
         if (CONV) {
             // Eq. 4 against the previous iterate, which the state in global
             // memory holds in this mode (it is rewritten every iteration)
-            __syncthreads();
             const float* Xf = (const float*)X;
             float lsum = 0.0f;
-            constexpr int PER = (1 << LOG2L) / kResThreads;  // 2 .. 32 samples per thread
-            constexpr int G = PER < 8 ? PER : 8;              // loads issued before stores
+            constexpr int PER = L / TH;             // 2 .. 32 samples per thread
+            constexpr int G = PER < 8 ? PER : 8;    // loads issued before stores
 #pragma unroll
             for (int g0 = 0; g0 < PER; g0 += G) {
                 float xn[G], xo[G];
 #pragma unroll
                 for (int j = 0; j < G; ++j) {
-                    const int m = threadIdx.x + (g0 + j) * kResThreads;
+                    const int m = threadIdx.x + (g0 + j) * TH;
                     xo[j] = xg[m];
                     xn[j] = Xf[fsw(m)];
                 }
 #pragma unroll
                 for (int j = 0; j < G; ++j) {
                     lsum += ln_ratio_sq(xn[j], xo[j]);
-                    xg[threadIdx.x + (g0 + j) * kResThreads] = xn[j];
+                    xg[threadIdx.x + (g0 + j) * TH] = xn[j];
                 }
             }
             const double delta = conv_delta(cta_sum(lsum, red), (double)L);
@@ -406,7 +463,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident_cta(const ResArgs a
         }
     }
     float2* xo2 = (float2*)xg;
-    for (int m = threadIdx.x; m < M; m += kResThreads) xo2[m] = z[swz(m)];
+    for (int m = threadIdx.x; m < M; m += TH) xo2[m] = z[swz(m)];
 }
 
 // ------------------------------------------------------------- clusters
@@ -538,10 +595,10 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kResThreads, 1) k_re
         // local stable sort of the block's keys (positions are local)
         uint32_t* kU = (uint32_t*)U;
         uint32_t* kV = (uint32_t*)V;
-        radix_pass<kResMaxLog2, true, false>((const float*)V, nullptr, kU, nullptr, ia, nullptr, s, 0, wh, dbase, wsum);
-        radix_pass<kResMaxLog2, false, false>(nullptr, kU, kV, ia, ib, nullptr, s, 8, wh, dbase, wsum);
-        radix_pass<kResMaxLog2, false, false>(nullptr, kV, kU, ib, ia, nullptr, s, 16, wh, dbase, wsum);
-        radix_pass<kResMaxLog2, false, false>(nullptr, kU, kV, ia, ib, nullptr, s, 24, wh, dbase, wsum);
+        radix_pass<kResMaxLog2, true>((const float*)V, nullptr, kU, nullptr, ia, 0, wh, dbase, wsum);
+        radix_pass<kResMaxLog2, false>(nullptr, kU, kV, ia, ib, 8, wh, dbase, wsum);
+        radix_pass<kResMaxLog2, false>(nullptr, kV, kU, ib, ia, 16, wh, dbase, wsum);
+        radix_pass<kResMaxLog2, false>(nullptr, kU, kV, ia, ib, 24, wh, dbase, wsum);
         // sorted keys in kV, positions in ib; publish the keys
         for (int p = threadIdx.x; p < L; p += kResThreads) __stcg(gk + me * L + p, kV[p]);
         cl.sync();  // every sorted block published
@@ -625,8 +682,9 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kResThreads, 1) k_re
 }
 
 template <int LOG2L>
-void launch_cta(const ResArgs& a, int ncurves, size_t smem, cudaStream_t st)
+void launch_cta(const ResArgs& a, int ncurves, cudaStream_t st)
 {
+    constexpr size_t smem = CtaShape<LOG2L>::BYTES;
     if (a.conv.delta) k_resident_cta<LOG2L, true><<<ncurves, kResThreads, smem, st>>>(a);
     else k_resident_cta<LOG2L, false><<<ncurves, kResThreads, smem, st>>>(a);
 }
@@ -638,8 +696,7 @@ void launch_cluster(const ResArgs& a, int ncurves, size_t smem, cudaStream_t st)
     else k_resident_cluster<C, false><<<ncurves * C, kResThreads, smem, st>>>(a);
 }
 
-// Shared memory of the fused kernels at their longest one-CTA length (the
-// cluster kernels hold the same per CTA).
+// Shared memory of a cluster kernel's CTA, more than any one-CTA kernel takes.
 constexpr size_t kResSmemMax = 12 * ((size_t)1 << kResMaxLog2) + kWhBytes + kTwBytes;
 
 template <typename F>
@@ -673,11 +730,11 @@ cudaError_t resident_kernel_attributes()
 }
 
 // Path table of the auto mode: the one-CTA fused kernel from 2^10 to 2^12,
-// the multi-kernel path above (autotune.py on GB300, 2^26 samples x 20
-// iterations, sample*iter/s fused vs multi-kernel: 2^12 3.79e10 vs 2.51e10,
-// 2^13 4.22e10 vs 4.48e10, 2^14 3.99e10 vs 4.87e10, 2^15 2.20e10 for the
-// 2-CTA cluster kernel vs 4.92e10).  With the LSD argsort the crossover was
-// 2^14.  LC_RESIDENT_MAX_LOG2 (up to 14 for the one-CTA kernel) moves it;
+// the multi-kernel path above (2^26 samples x 20 iterations, sample*iter/s
+// fused vs multi-kernel: 2^10 4.8e10 vs 4.1e10, 2^11 7.1e10 vs 4.9e10, 2^12
+// 8.7e10 vs 4.5e10, 2^13 6.9e10 vs 4.4e10, 2^14 4.5e10 vs 4.7e10, 2^15 2.2e10
+// for the 2-CTA cluster kernel vs 4.9e10).  The two paths' transforms round
+// differently, so 2^13 stays where its results have been.  LC_RESIDENT_MAX_LOG2 (up to 14 for the one-CTA kernel) moves it;
 // LC_PATH=resident also runs the cluster kernels at 2^15 and 2^16.
 bool resident_supported(const Plan& p, uint32_t log2n)
 {
@@ -708,20 +765,18 @@ void launch_resident(const Plan& p, const ClassInfo& k, uint32_t n_it, cudaStrea
     a.log2n = k.log2n;
     a.conv = conv_of(p);
     const int C = k.log2n <= kResMaxLog2 ? 1 : 1 << (k.log2n - kResMaxLog2);
-    const size_t L = ((size_t)1 << k.log2n) / C;
-    const size_t smem = 12 * L + kWhBytes + kTwBytes;
     if (C == 1) {
         switch (k.log2n) {
-        case 10: launch_cta<10>(a, k.ncurves, smem, st); break;
-        case 11: launch_cta<11>(a, k.ncurves, smem, st); break;
-        case 12: launch_cta<12>(a, k.ncurves, smem, st); break;
-        case 13: launch_cta<13>(a, k.ncurves, smem, st); break;
-        default: launch_cta<14>(a, k.ncurves, smem, st); break;
+        case 10: launch_cta<10>(a, k.ncurves, st); break;
+        case 11: launch_cta<11>(a, k.ncurves, st); break;
+        case 12: launch_cta<12>(a, k.ncurves, st); break;
+        case 13: launch_cta<13>(a, k.ncurves, st); break;
+        default: launch_cta<14>(a, k.ncurves, st); break;
         }
     } else if (C == 2) {
-        launch_cluster<2>(a, k.ncurves, smem, st);
+        launch_cluster<2>(a, k.ncurves, kResSmemMax, st);
     } else {
-        launch_cluster<4>(a, k.ncurves, smem, st);
+        launch_cluster<4>(a, k.ncurves, kResSmemMax, st);
     }
     if (launches) ++*launches;
 }
