@@ -55,6 +55,7 @@ lc_status prepare_kernels(int device)
     cudaError_t e = fft_kernel_attributes();
     if (e == cudaSuccess) e = resident_kernel_attributes();
     if (e == cudaSuccess) e = bucket_kernel_attributes();
+    if (e == cudaSuccess) e = rank_kernel_attributes();
     if (e != cudaSuccess) {
         set_error(std::string("kernel attributes: ") + cudaGetErrorString(e));
         return LC_ERR_CUDA;
@@ -197,6 +198,7 @@ static lc_status plan_describe(const lc_job* jobs, size_t njobs, lc_precision pr
     for (auto& k : p->classes) {
         k.ncurves = (int)k.h_curves.size();
         k.bucket = bucket_on && bucket_supported(prec, k.log2n);
+        k.rank_cta = bucket_on && rank_cta_supported(prec, k.log2n);
         k.radices = fft_radices(k.log2n - 1);
         const size_t n = 1ull << k.log2n;
         k.tile_len = (int)std::min<size_t>(n, kSortTile);
@@ -228,6 +230,7 @@ static PlanLayout plan_layout(Plan& P, bool ext)
     for (auto& k : p->classes) {
         const size_t n = 1ull << k.log2n;
         if (k.bucket) auxb += align_up(bucket_aux_words(k.log2n, k.ncurves) * 4, 256);
+        if (k.rank_cta && !k.resident) auxb += align_up((size_t)k.ncurves * kRankBounds * 4, 256);
         k.hist_off = hist;  hist += (size_t)k.ncurves * k.tiles_per_curve * 256;
         k.cbase_off = cbase; cbase += (size_t)k.ncurves * k.nchunks * 256;
         k.partial_off = partial; partial += (size_t)k.ncurves * spec_blocks_per_curve(k.log2n);
@@ -374,6 +377,10 @@ lc_status plan_create_ext(const lc_job* jobs, size_t njobs, lc_precision prec, i
         if (k.bucket) {
             k.d_aux = (uint32_t*)(base + aux_at);
             aux_at += align_up(bucket_aux_words(k.log2n, k.ncurves) * 4, 256);
+        }
+        if (k.rank_cta && !k.resident) {
+            k.d_bounds = (float*)(base + aux_at);
+            aux_at += align_up((size_t)k.ncurves * kRankBounds * 4, 256);
         }
         k.d_tw = base + tw_at;
         tw_at += align_up((((size_t)1 << k.log2n) / 2) * 2 * ts, 256);

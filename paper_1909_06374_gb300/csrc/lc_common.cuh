@@ -87,6 +87,10 @@ __device__ __forceinline__ double key_value(unsigned long long k)
     return __longlong_as_double((long long)((k & 0x8000000000000000ull) ? (k & 0x7fffffffffffffffull) : ~k));
 }
 
+// The value whose bits are stored in a key word.
+__device__ __forceinline__ float value_bits(uint32_t b) { return __uint_as_float(b); }
+__device__ __forceinline__ double value_bits(unsigned long long b) { return __longlong_as_double((long long)b); }
+
 // ------------------------------------------------------------ Philox4x32-10
 // Salmon, Moraes, Dror & Shaw (SC'11): ten rounds of the Philox-4x32 bijection
 // with multipliers 0xD2511F53 / 0xCD9E8D57 and Weyl key increments

@@ -32,6 +32,8 @@ struct ClassInfo {
     float* d_rx = nullptr;             // L2 exchange area of the cluster kernel (3 N floats per curve)
     bool bucket = false;               // argsort by the sample sort of lc_bucket.cu
     uint32_t* d_aux = nullptr;         // its splitters, bases and work items
+    bool rank_cta = false;             // ranked and sorted by one CTA per curve (lc_rank.cu)
+    float* d_bounds = nullptr;         // its segment bounds from the iteration before (may be null)
     int ntab = 0;                      // curves with a tabulated ERDF (Eq. 1 smooth, Eq. 2)
     int* d_tab_curves = nullptr;       // their curve indices (device)
     std::vector<int> h_tab_curves;
@@ -272,6 +274,14 @@ void launch_bucket_argsort(const Plan& p, const ClassInfo& k, const void* src, v
 void launch_bucket_argsort(const Plan& p, const std::vector<const ClassInfo*>& ks,
                            const std::vector<const void*>& srcs, void* x_out, bool gated, bool presampled,
                            cudaStream_t st, uint64_t* launches, KernelTimes* kt);
+// one CTA per curve (lc_rank.cu): classes with ClassInfo::rank_cta
+constexpr int kRankBounds = 260;  // floats per curve of ClassInfo::d_bounds
+bool rank_cta_supported(lc_precision prec, uint32_t log2n);
+cudaError_t rank_kernel_attributes();
+// values: the sorted values of src to s; else x_out[perm[r]] = s[r] (x_out
+// default the state)
+template <typename T> void launch_rank_cta(const Plan& p, const ClassInfo& k, const void* src, bool values,
+                                           void* x_out, bool gated, cudaStream_t st);
 // where the inverse transform's last pass writes the class's samples of
 // x_adj (curve ci at + ci bucket_curve_words(log2n) floats), and the shift of
 // their complex index (PassArgs::smp_shift)

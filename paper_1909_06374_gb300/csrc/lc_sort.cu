@@ -46,10 +46,6 @@ __device__ __forceinline__ bool curve_active(const SortArgs& a, int c)
     return !a.d_iter || (uint32_t)(*a.d_iter) < a.eff_iters[c];
 }
 
-// Key bits of a value stored as T, reinterpreted from the key word.
-__device__ __forceinline__ float value_bits(uint32_t b) { return __uint_as_float(b); }
-__device__ __forceinline__ double value_bits(unsigned long long b) { return __longlong_as_double((long long)b); }
-
 // Exclusive scan of v over the 256 threads of a block (all threads call it).
 __device__ __forceinline__ uint32_t block_exclusive_scan256(uint32_t v, uint32_t* wsum)
 {
@@ -602,6 +598,11 @@ void launch_sort(const Plan& p, const std::vector<const ClassInfo*>& ks, const s
         if (mode == kSortArgsortScatter && ks[i]->bucket) {
             bk.push_back(ks[i]);
             bsrc.push_back(srcs[i]);
+        } else if (ks[i]->rank_cta) {
+            if (kt) kt->begin(kGroupSortScatter, st);
+            launch_rank_cta<T>(p, *ks[i], srcs[i], mode == kSortKeysToValues, x_out, gated, st);
+            if (kt) kt->end(st);
+            if (launches) ++*launches;
         } else {
             rk.push_back(ks[i]);
             rsrc.push_back(srcs[i]);
