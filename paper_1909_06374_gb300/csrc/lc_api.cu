@@ -232,6 +232,7 @@ static PlanLayout plan_layout(Plan& P, bool ext)
         if (k.bucket) auxb += align_up(bucket_aux_words(k.log2n, k.ncurves) * 4, 256);
         if (k.rank_cta && !k.resident) auxb += align_up((size_t)k.ncurves * kRankBounds * 4, 256);
         k.hist_off = hist;  hist += (size_t)k.ncurves * k.tiles_per_curve * 256;
+        if (k.log2n >= kSortPlaceMinLog2) auxb += align_up((size_t)k.ncurves * 256 * 4, 256);
         k.cbase_off = cbase; cbase += (size_t)k.ncurves * k.nchunks * 256;
         k.partial_off = partial; partial += (size_t)k.ncurves * spec_blocks_per_curve(k.log2n);
         twb += align_up((n / 2) * 2 * ts, 256);
@@ -382,6 +383,10 @@ lc_status plan_create_ext(const lc_job* jobs, size_t njobs, lc_precision prec, i
             k.d_bounds = (float*)(base + aux_at);
             aux_at += align_up((size_t)k.ncurves * kRankBounds * 4, 256);
         }
+        if (k.log2n >= kSortPlaceMinLog2) {
+            k.d_cursor = (uint32_t*)(base + aux_at);
+            aux_at += align_up((size_t)k.ncurves * 256 * 4, 256);
+        }
         k.d_tw = base + tw_at;
         tw_at += align_up((((size_t)1 << k.log2n) / 2) * 2 * ts, 256);
         twb += align_up((((size_t)1 << k.log2n) / 2) * 2 * ts, 256);
@@ -432,6 +437,10 @@ lc_status plan_create_ext(const lc_job* jobs, size_t njobs, lc_precision prec, i
     if (p->ntab && (e = cudaMemcpyAsync(p->d_tab_curves, tab_all.data(), sizeof(int) * tab_all.size(),
                                         cudaMemcpyHostToDevice, p->stream)) != cudaSuccess)
         return fail("upload table curves", e);
+    for (auto& k : p->classes) {
+        if (k.d_cursor && (e = cudaMemsetAsync(k.d_cursor, 0, (size_t)k.ncurves * 256 * sizeof(uint32_t), p->stream)) !=
+                              cudaSuccess) return fail("clear cursors", e);
+    }
     lc_status st = prec == LC_FP32 ? build_tables<float>(*p) : build_tables<double>(*p);
     if (st != LC_OK) return fail("twiddle tables", cudaGetLastError());
     if ((e = cudaStreamSynchronize(p->stream)) != cudaSuccess) return fail("plan sync", e);

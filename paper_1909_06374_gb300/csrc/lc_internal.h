@@ -34,6 +34,7 @@ struct ClassInfo {
     uint32_t* d_aux = nullptr;         // its splitters, bases and work items
     bool rank_cta = false;             // ranked and sorted by one CTA per curve (lc_rank.cu)
     float* d_bounds = nullptr;         // its segment bounds from the iteration before (may be null)
+    uint32_t* d_cursor = nullptr;      // position-bucket cursors of the long curves' last sort pass
     int ntab = 0;                      // curves with a tabulated ERDF (Eq. 1 smooth, Eq. 2)
     int* d_tab_curves = nullptr;       // their curve indices (device)
     std::vector<int> h_tab_curves;
@@ -234,6 +235,11 @@ template <typename T> void launch_fft_iteration(const Plan& p, const std::vector
 template <typename T> void launch_spectral_tk(const Plan& p, const ClassInfo& k, void* Zp, cudaStream_t st);
 
 // sort stage (lc_sort.cu)
+// shortest length whose argsort stores its result by position buckets (the
+// state, 256 MB in FP32, no longer fits the 129 MB L2; 2^28 samples, ms per
+// iteration direct / by buckets: 2^24 11.7 / 12.2, 2^25 12.6 / 12.5, 2^26
+// 14.3 / 12.9)
+constexpr uint32_t kSortPlaceMinLog2 = 26;
 constexpr int kSortTile = 2048;
 constexpr int kScanChunk = 32;
 enum SortMode { kSortArgsortScatter = 1, kSortKeysToValues = 2 };

@@ -39,12 +39,25 @@ struct SortArgs {
     int nchunks;
     int tile_len;
     int shift;
+    uint32_t* cursor;      // kSortArgsortPlace: [ncurves][256] pairs stored of each position bucket
+    int pshift;            // its position bucket: position >> pshift (256 buckets)
 };
+
+// Last pass of an argsort of long curves, in two steps: the new values go with
+// their positions to 256 buckets of positions (kSortArgsortPlace), and
+// k_sort_place stores them.  x[position] = s[rank] straight from the pass
+// (kSortArgsortScatter) spreads 4-byte stores over the whole state: once that
+// exceeds L2 each one moves a 32-byte sector in and out of HBM.
+constexpr int kSortArgsortPlace = 3;
 
 __device__ __forceinline__ bool curve_active(const SortArgs& a, int c)
 {
     return !a.d_iter || (uint32_t)(*a.d_iter) < a.eff_iters[c];
 }
+
+// Bits of a value as a key word.
+__device__ __forceinline__ uint32_t value_key(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ unsigned long long value_key(double v) { return (unsigned long long)__double_as_longlong(v); }
 
 // Exclusive scan of v over the 256 threads of a block (all threads call it).
 __device__ __forceinline__ uint32_t block_exclusive_scan256(uint32_t v, uint32_t* wsum)
@@ -234,6 +247,9 @@ constexpr int kSlots = kSortTile / kSortThreads;  // elements per thread of a fu
 // the curve is gb[d] + (count of d in earlier warps) + (rank in its warp), and
 // the element writes x[position] = s[rank] straight from registers (the
 // stores are scattered anyway), with no shared-memory placement.
+// kSortArgsortPlace: the pair (s[rank], position) goes to its position bucket:
+// counted by shared-memory atomics, a run per bucket reserved at the bucket's
+// cursor (the order inside a bucket is arbitrary), stored coalesced.
 // src_t / src_k / src_v point at the tile's first value / key / position.
 // FULL: a tile of kSortTile elements (no bounds tests).  THREADS >= 256 (one
 // thread per digit in the per-digit steps).  Expects wcnt zeroed and gb set
@@ -244,7 +260,7 @@ __device__ __forceinline__ void sort_tile(const SortArgs& a, const T* __restrict
                                           const uint32_t* __restrict__ src_v, void* kout, uint32_t* vout, int shift,
                                           uint64_t off, uint32_t e0, int tl, typename key_of<T>::type* sk,
                                           uint32_t* sv, uint32_t (*wcnt)[256], uint32_t* ldstart, uint32_t* gb,
-                                          uint32_t* wsum)
+                                          uint32_t* wsum, int cursor_row)
 {
     using K = typename key_of<T>::type;
     constexpr int WARPS = THREADS / 32;
@@ -319,6 +335,47 @@ __device__ __forceinline__ void sort_tile(const SortArgs& a, const T* __restrict
         for (int e = 0; e < SLOTS; ++e)
             if (rk[e] != 0xffffffffu) x_out[val[e]] = xn[e];
         __syncthreads();
+        return;
+    }
+    if (MODE == kSortArgsortPlace) {
+        static_assert(MODE != kSortArgsortPlace || THREADS == 256, "one thread per bucket");
+        ldstart[tid] = 0u;
+        __syncthreads();
+        const T* __restrict__ s_in = (const T*)a.s_in + off;
+#pragma unroll
+        for (int e = 0; e < SLOTS; ++e) {
+            if (rk[e] != 0xffffffffu) {
+                const uint32_t d = info[e] & 255u;
+                key[e] = value_key(s_in[gb[d] + wcnt[warp][d] + rk[e]]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < SLOTS; ++e)
+            if (rk[e] != 0xffffffffu) rk[e] = atomicAdd(&ldstart[val[e] >> a.pshift], 1u);
+        __syncthreads();
+        const uint32_t cnt = ldstart[tid];
+        uint32_t* cur = a.cursor + (size_t)(cursor_row)*256 + tid;
+        const uint32_t at = ((uint32_t)tid << a.pshift) + (cnt ? atomicAdd(cur, cnt) : 0u);
+        const uint32_t ls = block_exclusive_scan256(cnt, wsum);  // a barrier: every thread has read its count
+        ldstart[tid] = ls;
+        gb[tid] = at - ls;
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < SLOTS; ++e) {
+            if (rk[e] != 0xffffffffu) {
+                const uint32_t lp = ldstart[val[e] >> a.pshift] + rk[e];
+                sk[lp] = key[e];
+                sv[lp] = val[e];
+            }
+        }
+        __syncthreads();
+        K* __restrict__ kdst = (K*)kout + off;
+        uint32_t* __restrict__ vdst = vout + off;
+        for (int i = tid; i < tl; i += THREADS) {
+            const uint32_t v = sv[i], dest = gb[v >> a.pshift] + (uint32_t)i;
+            kdst[dest] = sk[i];
+            vdst[dest] = v;
+        }
         return;
     }
     // the tile's digit starts (digits are threads 0..255)
@@ -398,10 +455,39 @@ __global__ void __launch_bounds__(THREADS, MINB) k_sort_scatter(const __grid_con
     const uint32_t* src_v = a.vals_in + off + e0;
     if (a.tile_len == kSortTile)
         sort_tile<T, FIRST, MODE, true, THREADS>(a, src_t, src_k, src_v, a.keys_out, a.vals_out, a.shift, off, e0,
-                                                 a.tile_len, sk, sv, wcnt, ldstart, gb, wsum);
+                                                 a.tile_len, sk, sv, wcnt, ldstart, gb, wsum, ci);
     else
         sort_tile<T, FIRST, MODE, false, THREADS>(a, src_t, src_k, src_v, a.keys_out, a.vals_out, a.shift, off, e0,
-                                                  a.tile_len, sk, sv, wcnt, ldstart, gb, wsum);
+                                                  a.tile_len, sk, sv, wcnt, ldstart, gb, wsum, ci);
+}
+
+// The second step of kSortArgsortPlace: one tile of kSortTile pairs per block,
+// x[position] = value.  The blocks at work share a few position buckets, whose
+// N / 256 samples lie in L2 while their stores arrive.
+template <typename T, bool MULTI>
+__global__ void __launch_bounds__(kSortThreads) k_sort_place(const __grid_constant__ LaunchSet<SortArgs> set)
+{
+    uint32_t blk;
+    const SortArgs& a = set.pick<MULTI>(blk);
+    using K = typename key_of<T>::type;
+    const int ci = (int)blk / a.tpc;
+    const int c = a.cls_curves[ci];
+    if (!curve_active(a, c)) return;
+    if ((int)blk % a.tpc == 0) a.cursor[(size_t)ci * 256 + threadIdx.x] = 0u;  // for the next argsort
+    const uint64_t off = a.curves[c].off;
+    const uint64_t e0 = off + (uint64_t)((int)blk % a.tpc) * kSortTile + threadIdx.x;
+    const K* __restrict__ k = (const K*)a.keys_out + e0;
+    const uint32_t* __restrict__ v = a.vals_out + e0;
+    T* __restrict__ x = (T*)a.x_out + off;
+    K q[kSortTile / kSortThreads];
+    uint32_t p[kSortTile / kSortThreads];
+#pragma unroll
+    for (int e = 0; e < kSortTile / kSortThreads; ++e) {
+        q[e] = k[e * kSortThreads];
+        p[e] = v[e * kSortThreads];
+    }
+#pragma unroll
+    for (int e = 0; e < kSortTile / kSortThreads; ++e) x[p[e]] = value_bits(q[e]);
 }
 
 // Eq. 4 (Sec. 3.2.2) from the two iterates, both in natural order: one tile
@@ -511,7 +597,9 @@ static void scatter_v(int mode, const LaunchSet<SortArgs>& s, uint32_t g, cudaSt
     constexpr int TH = 256, MB = 5;
     if (mode == 0) k_sort_scatter<T, FIRST, 0, TH, MB, MULTI><<<g, TH, 0, st>>>(s);
     else if (mode == kSortArgsortScatter) k_sort_scatter<T, FIRST, kSortArgsortScatter, TH, MB, MULTI><<<g, TH, 0, st>>>(s);
-    else k_sort_scatter<T, FIRST, kSortKeysToValues, TH, MB, MULTI><<<g, TH, 0, st>>>(s);
+    else if (mode == kSortArgsortPlace) {
+        if constexpr (!FIRST) k_sort_scatter<T, FIRST, kSortArgsortPlace, TH, MB, MULTI><<<g, TH, 0, st>>>(s);
+    } else k_sort_scatter<T, FIRST, kSortKeysToValues, TH, MB, MULTI><<<g, TH, 0, st>>>(s);
 }
 
 template <typename T, bool FIRST>
@@ -587,6 +675,32 @@ static int launch_scan(const std::vector<SortArgs>& args, cudaStream_t st)
     return n;
 }
 
+// The last pass over the classes: those with cursors in two steps, unless the
+// new state goes where the pairs would (the convergence test's key buffer B).
+template <typename T>
+static int launch_last_pass(const Plan& p, const std::vector<const ClassInfo*>& ks, SortMode mode,
+                            const std::vector<SortArgs>& args, const std::vector<uint32_t>& blocks, cudaStream_t st)
+{
+    std::vector<SortArgs> one, two;
+    std::vector<uint32_t> b_one, b_two;
+    for (size_t i = 0; i < ks.size(); ++i) {
+        const bool place = mode == kSortArgsortScatter && ks[i]->d_cursor && args[i].x_out != p.d_keysB;
+        (place ? two : one).push_back(args[i]);
+        (place ? b_two : b_one).push_back(blocks[i]);
+        if (place) {
+            two.back().cursor = ks[i]->d_cursor;  // zero: the plan's memset, then k_sort_place
+            two.back().pshift = (int)ks[i]->log2n - 8;
+        }
+    }
+    int n = launch_scatter<T, false>((int)mode, one, b_one, st);
+    n += launch_scatter<T, false>(kSortArgsortPlace, two, b_two, st);
+    n += for_launch_sets(two, b_two, [&](const LaunchSet<SortArgs>& s, uint32_t g, bool multi) {
+        if (multi) k_sort_place<T, true><<<g, kSortThreads, 0, st>>>(s);
+        else k_sort_place<T, false><<<g, kSortThreads, 0, st>>>(s);
+    });
+    return n;
+}
+
 template <typename T>
 void launch_sort(const Plan& p, const std::vector<const ClassInfo*>& ks, const std::vector<const void*>& srcs,
                  SortMode mode, bool gated, cudaStream_t st, uint64_t* launches, void* x_out, KernelTimes* kt,
@@ -649,10 +763,10 @@ void launch_sort(const Plan& p, const std::vector<const ClassInfo*>& ks, const s
         n += launch_hist<T>(first, args, st);
         n += launch_scan(args, st);
         if (kt) kt->end(st);
-        const int m = last ? (int)mode : 0;
         if (kt) kt->begin(kGroupSortScatter, st);
-        if (first) n += launch_scatter<T, true>(m, args, blocks, st);
-        else n += launch_scatter<T, false>(m, args, blocks, st);
+        if (first) n += launch_scatter<T, true>(0, args, blocks, st);
+        else if (!last) n += launch_scatter<T, false>(0, args, blocks, st);
+        else n += launch_last_pass<T>(p, rk, mode, args, blocks, st);
         if (kt) kt->end(st);
     }
     if (launches) *launches += (uint64_t)n;
