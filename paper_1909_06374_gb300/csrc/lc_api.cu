@@ -574,19 +574,34 @@ static lc_status run_iterations_impl(Plan& p, uint32_t override_iters, uint32_t 
     bool any_multi = false;
     for (auto& k : p.classes) any_multi |= !k.resident;
     if (any_multi && n_it > 0) {
-        if (!p.iter_graph) {
+        auto instantiate = [&](cudaGraphExec_t& exec, uint32_t iters) -> lc_status {
+            if (exec) return LC_OK;
             cudaGraph_t g = nullptr;
             uint64_t per = 0;
             LC_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            enqueue_iteration<T>(p, st, &per);
+            for (uint32_t q = 0; q < iters; ++q) {
+                per = 0;
+                enqueue_iteration<T>(p, st, &per);
+            }
             cudaError_t e = cudaStreamEndCapture(st, &g);
             if (e != cudaSuccess) { set_error(std::string("graph capture: ") + cudaGetErrorString(e)); return LC_ERR_CUDA; }
-            e = cudaGraphInstantiate(&p.iter_graph, g, 0);
+            e = cudaGraphInstantiate(&exec, g, 0);
             cudaGraphDestroy(g);
             if (e != cudaSuccess) { set_error(std::string("graph instantiate: ") + cudaGetErrorString(e)); return LC_ERR_CUDA; }
             p.launches_per_iter = per;
+            return LC_OK;
+        };
+        uint32_t it = 0;
+        if (p.total <= kGraphSamples && n_it >= 2 * kGraphIters) {
+            const lc_status gs = instantiate(p.iter_graphs, kGraphIters);
+            if (gs != LC_OK) return gs;
+            for (; it + kGraphIters <= n_it; it += kGraphIters) LC_CK(cudaGraphLaunch(p.iter_graphs, st));
         }
-        for (uint32_t it = 0; it < n_it; ++it) LC_CK(cudaGraphLaunch(p.iter_graph, st));
+        if (it < n_it) {
+            const lc_status gs = instantiate(p.iter_graph, 1);
+            if (gs != LC_OK) return gs;
+        }
+        for (; it < n_it; ++it) LC_CK(cudaGraphLaunch(p.iter_graph, st));
         *launches += (uint64_t)n_it * p.launches_per_iter;
     } else if (n_it > 0) {
         launch_iter_add(p, n_it, st);
@@ -623,6 +638,7 @@ void plan_free(Plan* p)
         DeviceGuard g(p->device);
         cudaStreamSynchronize(p->stream);
         if (p->iter_graph) cudaGraphExecDestroy(p->iter_graph);
+        if (p->iter_graphs) cudaGraphExecDestroy(p->iter_graphs);
         if (p->ext) {
             cudaFreeAsync(p->arena, p->stream);
             cudaStreamSynchronize(p->stream);
@@ -894,10 +910,10 @@ lc_status lc_plan_set_convergence(lc_plan plan, const double* thresholds, uint32
     LC_CK(cudaMemcpyAsync((void*)plan->conv.thr, thr.data(), nc * 8, cudaMemcpyHostToDevice, plan->stream));
     launch_conv_reset(*plan, plan->stream);
     LC_CK(cudaStreamSynchronize(plan->stream));
-    // the captured iteration graph has the kernels of the other mode
-    if (plan->iter_graph) {
-        cudaGraphExecDestroy(plan->iter_graph);
-        plan->iter_graph = nullptr;
+    // the captured iteration graphs have the kernels of the other mode
+    for (cudaGraphExec_t* exec : {&plan->iter_graph, &plan->iter_graphs}) {
+        if (*exec) cudaGraphExecDestroy(*exec);
+        *exec = nullptr;
     }
     return LC_OK;
 }

@@ -83,7 +83,8 @@ struct Plan {
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     cudaEvent_t t_setup0 = nullptr, t_setup1 = nullptr, t_it0 = nullptr, t_it1 = nullptr;
     bool timed_setup = false, timed_iter = false;
-    cudaGraphExec_t iter_graph = nullptr;
+    cudaGraphExec_t iter_graph = nullptr;   // one iteration
+    cudaGraphExec_t iter_graphs = nullptr;  // kGraphIters of them (small plans)
     uint64_t launches_per_iter = 0;
     uint64_t last_launches = 0;
     bool setup_done = false;
@@ -98,6 +99,13 @@ struct Plan {
     ConvDev conv{};
     size_t conv_part = 0;        // doubles in conv.part
 };
+
+// Iterations per graph of a small plan (at most kGraphSamples samples): the gap
+// between two graphs of a stream is about 3 us, of the 49 us that an iteration
+// of one 2^17 curve takes; larger plans have nothing to gain for the longer
+// instantiation.
+constexpr uint32_t kGraphIters = 4;
+constexpr size_t kGraphSamples = (size_t)1 << 20;
 
 // CUDA events around the kernel groups of one profiled iteration.
 enum KernelGroup {
