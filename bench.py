@@ -59,10 +59,14 @@ ITER_DRAM_CAPTURE_CURRENT = False
 # 1 + 8, finish 8 + 4 + 4, bucket byte written 1
 BUCKET_SORT_BYTES_PER_ELEMENT = 34
 SAMPLE_SORT_LOG2 = (13, 20)  # FP32 lengths on the sample sort
+RANK_CTA_LOG2 = {4: (10, 12), 8: (10, 14)}  # lengths one CTA ranks whole on the multi-kernel path, by sample size
+RANK_CTA_VALUES = 3          # values it moves per element: the value, its new one read and written
+SORT_PLACE_LOG2 = 26         # lengths from here on store the argsort's result by position buckets:
+                             # the pair (value, position) once more written and read
 FUSED_LOG2 = (10, 14)        # FP32 lengths the one-CTA fused kernel can take
 
 
-def scheduled_bytes_per_sample_iter(jobs, esize, fused_elements):
+def scheduled_bytes_per_sample_iter(jobs, esize, fused_elements, radix_only=True):
     """HBM bytes the scheduled kernels move per sample-iteration (reads +
     writes at their algorithmic sizes), averaged over the batch's
     sample-iterations, beside the 14 B floor (28 B in FP64).  Multi-kernel
@@ -72,7 +76,9 @@ def scheduled_bytes_per_sample_iter(jobs, esize, fused_elements):
     passes each way and the spectral kernel), each 2 esize B per sample, plus
     the amplitudes (esize / 2 B per sample); then the argsort: the sample
     sort's 34 B per element, or the radix passes with their histograms
-    (FP32: 4 x 4 + 60 = 76 B; FP64: 8 x 8 + 192 = 256 B).  Fused curves touch
+    (FP32: 4 x 4 + 60 = 76 B; FP64: 8 x 8 + 192 = 256 B).  Without radix_only:
+    three values per element where one CTA ranks a curve whole, and the
+    position buckets of the longest radix-sorted curves (16 and 24 B).  Fused curves touch
     HBM once per launch of all iterations: 14 B per sample (FP32) / iterations.
     The fused curves are those of 2^10..2^top for the top length whose
     samples add up to the plan's fused samples (the path table's crossover,
@@ -106,9 +112,12 @@ def scheduled_bytes_per_sample_iter(jobs, esize, fused_elements):
             fft = kernels * 2 * esize + esize / 2
             if fp32 and SAMPLE_SORT_LOG2[0] <= log2n <= SAMPLE_SORT_LOG2[1]:
                 sort = BUCKET_SORT_BYTES_PER_ELEMENT
+            elif not radix_only and RANK_CTA_LOG2[esize][0] <= log2n <= RANK_CTA_LOG2[esize][1]:
+                sort = RANK_CTA_VALUES * esize
             else:
                 passes = esize  # 8-bit digits of esize-byte keys
                 sort = passes * esize + SORT_BYTES_PER_ELEMENT[esize]  # histograms + scatter passes
+                sort += 2 * (esize + 4) if not radix_only and log2n >= SORT_PLACE_LOG2 else 0
             per = fft + sort
         tot_b += per * n * iters
         tot_si += n * iters
@@ -446,17 +455,24 @@ def gpu_line(args, workload, steps, warmup, dist, e2e_on, cpu_on, extra=False):
             dominant = "sort_scatter"
             launches_k = max(1, prof["scatter_launches"])
             nb = prof.get("bucket_elements", 0)
-            nr = prof["sorted_elements"] - nb
+            lo, hi = RANK_CTA_LOG2[esize]
+            nc = sum(1 << int(j["log2n"]) for j in jobs if lo <= int(j["log2n"]) <= hi) if not prof["fused_elements"] else 0
+            nr = prof["sorted_elements"] - nb - nc
             # every element of a radix-sorted class goes through all passes; every
             # element of a sample-sorted class through the bucket scatter and finish
-            per_launch_bytes = (SORT_BYTES_PER_ELEMENT[esize] * nr + BUCKET_SCATTER_BYTES_PER_ELEMENT * nb) / launches_k
+            per_launch_bytes = (SORT_BYTES_PER_ELEMENT[esize] * nr + BUCKET_SCATTER_BYTES_PER_ELEMENT * nb +
+                                RANK_CTA_VALUES * esize * nc) / launches_k
             if nb and not nr:
                 kernel = "k_bk_scatter + k_bk_finish (sample-sort argsort: bucket scatter and on-chip ranking)"
                 kernel_bytes_def = f"{BUCKET_SCATTER_BYTES_PER_ELEMENT} B per element (scatter 13 + finish 16)"
+            elif nc and not nr:
+                kernel = "k_rank_cta (one CTA ranks a curve on chip)"
+                kernel_bytes_def = f"{RANK_CTA_VALUES * esize} B per element (value, sorted draw, new state)"
             else:
                 kernel = "k_sort_scatter (radix passes of the argsort)" + (" and the sample-sort scatter" if nb else "")
                 kernel_bytes_def = (f"{SORT_BYTES_PER_ELEMENT[esize]} B per element per radix argsort (all passes), "
                                     f"{BUCKET_SCATTER_BYTES_PER_ELEMENT} B per sample-sorted element, "
+                                    f"{RANK_CTA_VALUES * esize} B per element that one CTA ranks, "
                                     "split evenly over the scatter launches")
         avg_ms = prof[dominant] / launches_k
         achieved = per_launch_bytes / (avg_ms / 1000.0) / 1e9
@@ -485,7 +501,7 @@ def gpu_line(args, workload, steps, warmup, dist, e2e_on, cpu_on, extra=False):
                                     "traffic": ktraffic, "alg_bytes_definition": kernel_bytes_def},
                 "group_ms_one_iteration": {g: prof[g] for g in groups},
                 "scheduled_bytes_per_sample_iter": scheduled_bytes_per_sample_iter(jobs, esize,
-                                                                                   prof["fused_elements"]),
+                                                                                   prof["fused_elements"], radix_only=False),
                 "setup_ms": setup_ms}
 
         if args.post and not extra:

@@ -192,7 +192,8 @@ LC_API lc_status lc_set_state(lc_plan plan, const void* in_x, void* stream);
  * s_c are the curve's sorted draws and perm_c the stable ascending argsort of
  * x_adj's curve c (ties, -0 = +0 included, keep the lower position first).
  * The plan's own sort path runs (the sample sort of FP32 curves of 2^13 ..
- * 2^20 samples, else the LSD radix passes).
+ * 2^20 samples, one CTA per curve at 2^10 .. 2^12 and, in FP64, 2^10 .. 2^14,
+ * else the LSD radix passes).
  *   x_adj: device pointer, sum_c N_c elements in the plan's precision and
  *          layout (curve c at the offset of lc_get_state); read only; values
  *          must not be NaN.
@@ -291,7 +292,8 @@ LC_API lc_status lc_structure_function(lc_plan plan, const void* x, const uint32
  *   group_ms[4] convergence test.
  * ngroups: entries of group_ms to fill (extra ones get 0).
  * counts (nullable, 4 entries): scatter spans timed (one per radix pass of
- * each radix-sorted class, one per sample-sorted class), samples of the
+ * each radix-sorted class, one per sample-sorted class and per class that one
+ * CTA per curve ranks), samples of the
  * multi-kernel classes, samples of the fused classes, samples of the
  * multi-kernel classes whose argsort is the sample sort.
  * The state advances by one iteration; the iteration counter restarts, so a

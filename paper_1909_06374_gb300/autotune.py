@@ -8,7 +8,8 @@ For every length in the range this sweep runs a uniform batch of about
 2^samples samples for `iters` iterations on each path, timed with CUDA events
 around the iteration stage (lc_plan_timing), and reports the crossover: the
 longest length up to which the fused kernels win at every length.  The
-library's auto mode uses the crossover measured on GB300 (2^12); the
+library's auto mode uses 2^12 (on GB300 the fused kernels now win at 2^13 as
+well, but those curves keep the path, hence the bits, they had); the
 environment variable LC_RESIDENT_MAX_LOG2 applies another one (read when a
 plan is created).  Results depend on the length, the precision and the path,
 so a different crossover changes the bits of the affected lengths (both paths

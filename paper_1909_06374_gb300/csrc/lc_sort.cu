@@ -9,7 +9,9 @@
 // (tile, digit) its output base, and a stable scatter that ranks the tile in
 // shared memory (ballot/match multisplit + per-warp counts) and writes each
 // digit's run with coalesced stores.  The last pass of an argsort writes
-// x[k] = s[rank] directly instead of the sorted pairs.
+// x[k] = s[rank] directly instead of the sorted pairs (from 2^26 on by way of
+// position buckets, k_sort_place).  Classes that lc_bucket.cu or lc_rank.cu
+// sort are handed over by launch_sort.
 #include <algorithm>
 
 #include "lc_internal.h"
