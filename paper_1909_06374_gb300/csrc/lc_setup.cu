@@ -25,15 +25,18 @@ constexpr int kSpecTile = kSpecBlock * kSpecPerThread;  // bins per block
 // Coefficient j of a curve (c = 1/(N dt f_br), nh = N/2).  y_j = f_j / f_br =
 // j c; Eq. 3 as 1 / (e^{a_lo ln y} + e^{a_hi ln y}) (one logarithm for both
 // terms); the amplitude sqrt(P/2) sqrt(-2 ln U1) as one square root: these are
-// the FP64 operations that the FP64-rate-bound kernels spend their time on.
+// the FP64 operations that the FP64-rate-bound kernels spend their time on
+// (conversions of 64-bit integers are among them: the uniforms, 2 U2 and j are
+// put together from their bits, with one exact subtraction each at most).
 __device__ __forceinline__ double2 tk_bin(const CurveDev& cv, double c, bool fixed, uint64_t j, uint64_t nh, double& P)
 {
     const uint4 w = philox(j, cv.curve_id, 0u, cv.seed);
-    const double U1 = unit_open(w.x, w.y), U2 = unit_open(w.z, w.w);
+    const double U1 = unit_open_fast(w.x, w.y), U2 = unit_open_fast(w.z, w.w);
     const double lu = fixed ? 0.0 : log(U1);  // rad^2 = -2 lu
     double sn, cs;
-    sincospi(2.0 * U2, &sn, &cs);
-    const double ly = log((double)j * c);
+    sincospi(__hiloint2double(__double2hiint(U2) + 0x100000, __double2loint(U2)), &sn, &cs);  // 2 U2, by its exponent
+    // j as a double: the low word of 2^52 + j, less 2^52 (j < 2^32, exact)
+    const double ly = log((__hiloint2double(0x43300000, (int)(uint32_t)j) - 0x1p52) * c);
     P = 1.0 / (exp(cv.a_lo * ly) + exp(cv.a_hi * ly));
     if (j < nh) {
         const double a = fixed ? sqrt(P) : sqrt(-P * lu);
