@@ -1,5 +1,6 @@
-"""Structure function of FP32 plans over the range of float: large and infinite
-samples, and the batches whose blocks take all lags of a curve."""
+"""Structure function and periodogram of FP32 plans over the range of float:
+large and infinite samples, bin powers at both ends, and the batches whose
+blocks take all lags of a curve."""
 import numpy as np
 import pytest
 
@@ -60,3 +61,20 @@ def test_structure_function_by_blocks_of_many_lags(curves, log2n, nlags):
         got = p.structure_function(torch.tensor(x.reshape(-1), device="cuda"), [int(l) for l in lags]).cpu().numpy()
     for c in {0, curves // 2, curves - 1}:
         np.testing.assert_allclose(got[c], oracle.structure_function(x[c].astype(np.float64), lags), rtol=SF_TOL)
+
+
+def test_bin_powers_keep_their_precision():
+    """x = (a, b, 0, 0, ...) has X_{N/4} = a - i b exactly (the transform's two
+    additions are of zeros), so that bin's power is (a^2 + b^2) 2 / N^2 to the
+    rounding of one FP64 addition."""
+    rng = np.random.default_rng(5)
+    ab = (rng.standard_normal((400, 2)) * 10.0 ** rng.uniform(-30, 30, (400, 1))).astype(np.float32)
+    ab = np.concatenate([ab, np.float32([[2.0 ** -46, 0], [0, 2.0 ** -46], [1, 0], [0, 0], [3, 4], [1e-40, 1e-42],
+                                         [2.0 ** -43, 2.0 ** -62], [1, 2.0 ** -12], [1, np.nan]])])
+    n = 16
+    x = np.zeros((len(ab), n), dtype=np.float32)
+    x[:, :2] = ab
+    with _plan(4, len(ab)) as p:
+        P = p.periodogram(torch.tensor(x.reshape(-1), device="cuda")).cpu().numpy().reshape(len(ab), n // 2 + 1)
+    a, b = ab.astype(np.float64).T
+    np.testing.assert_allclose(P[:, n // 4], (a * a + b * b) * (2.0 / n ** 2), rtol=2.0 ** -52)
