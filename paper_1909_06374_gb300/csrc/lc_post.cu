@@ -19,13 +19,13 @@ namespace lc {
 // E = (Z_k + conj Z_{M-k})/2, O = (Z_k - conj Z_{M-k})/(2i).
 // P_j = |X_j|^2 2/N^2 (Eq. A2) or |X_j|^2 2 dt N / X_0^2 (Eq. A4, X_0 = N mu).
 //
-// One block takes up to kPgPairs conjugate pairs of one curve.  A float bin's
+// One block takes `pairs` conjugate pairs of one curve (launch_periodogram).  A float bin's
 // power takes two FP64 operations (three for Eq. A4) of the 2 per clock and SM:
 // its conversions and Eq. A2's scale, a power of two, are put together from
 // bits.  2048 curves of 2^16 samples, transform included: 1.11 ms with FP64
 // conversions and scaling (Eq. A4, with a division per bin: 1.81), 0.976 (1.03)
 // with these.
-constexpr int kPgPairs = 4096;
+constexpr uint32_t kPgPairs = 4096;
 
 // (x^2 + y^2) 2^-sh, rounded once: a float's square is exact in FP64.
 __device__ __forceinline__ double power_of(float x, float y, int sh)
@@ -48,7 +48,7 @@ __device__ __forceinline__ double power_of(double x, double y, int sh)
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_periodogram(const int* __restrict__ cls_curves,
-                                                     const CurveDev* __restrict__ curves, int chunks, uint32_t log2M,
+                                                     const CurveDev* __restrict__ curves, uint32_t pairs, uint32_t log2M,
                                                      const void* __restrict__ tw, const void* __restrict__ Zin, int rms,
                                                      double* __restrict__ P)
 {
@@ -57,8 +57,9 @@ __global__ void __launch_bounds__(256) k_periodogram(const int* __restrict__ cls
     const uint32_t M = 1u << log2M;
     const double nd = 2.0 * (double)M;
     const V* __restrict__ rt = (const V*)tw;
-    const CurveDev& cv = curves[cls_curves[blockIdx.x / (uint32_t)chunks]];
-    const uint32_t k0 = blockIdx.x % (uint32_t)chunks * kPgPairs;
+    const uint32_t chunks = max(half / pairs, 1u);
+    const CurveDev& cv = curves[cls_curves[blockIdx.x / chunks]];
+    const uint32_t k0 = blockIdx.x % chunks * pairs;
     const V* __restrict__ Z = (const V*)Zin + (cv.off >> 1);
     double* __restrict__ out = P + cv.offh;
     // 2 / N^2 = 2^-sh, or the rms normalisation
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(256) k_periodogram(const int* __restrict__ cls
         const double v = power_of(x, y, sh);
         return rms ? v * scale : v;
     };
-    const uint32_t k1 = min(half, k0 + kPgPairs);
+    const uint32_t k1 = min(half, k0 + pairs);
 #pragma unroll 4
     for (uint32_t k = k0 + threadIdx.x; k < k1; k += 256) {
         if (k == 0) {
@@ -281,15 +282,26 @@ static void launch_structure(const Plan& p, const ClassInfo& k, int nlags, const
             k.d_curves, p.d_curves, k.ncurves, k.log2n, segs, nlags, p.d_lags, part, out);
 }
 
+// kPgPairs pairs per block where that gives two blocks per SM, fewer (down to
+// one per thread) where not: with their transform, one 2^16 FP32 curve
+// 18 us (kPgPairs per block: 29), 64 of 2^14 26 (35), one 2^16 FP64 curve 32 (56).
+template <typename T>
+static void launch_periodogram(const Plan& p, const ClassInfo& k, const void* Z, int rms, double* out, cudaStream_t st)
+{
+    const uint64_t half = 1ull << (k.log2n - 2);
+    uint32_t pairs = kPgPairs;
+    while (pairs > 256 && k.ncurves * half < 152ull * 2 * pairs) pairs /= 2;
+    const unsigned blocks = (unsigned)(k.ncurves * std::max<uint64_t>(half / pairs, 1));
+    k_periodogram<T><<<blocks, 256, 0, st>>>(k.d_curves, p.d_curves, pairs, k.log2n - 1, k.d_tw, Z, rms, out);
+}
+
 template <typename T>
 static void run_periodogram(Plan& p, const void* x, int rms, double* out, cudaStream_t st)
 {
     for (auto& k : p.classes) {
         // x is only read: the passes ping-pong between d_f and d_keysB
         void* Z = launch_fft<T>(p, k, false, const_cast<void*>(x), p.d_f, nullptr, false, st, nullptr, p.d_keysB);
-        const int chunks = std::max(1, (1 << (k.log2n - 2)) / kPgPairs);
-        k_periodogram<T><<<k.ncurves * chunks, 256, 0, st>>>(k.d_curves, p.d_curves, chunks, k.log2n - 1, k.d_tw, Z,
-                                                             rms, out);
+        launch_periodogram<T>(p, k, Z, rms, out, st);
     }
 }
 

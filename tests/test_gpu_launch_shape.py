@@ -1,0 +1,36 @@
+"""How the library's kernels are launched, from a trace of the launches."""
+import json
+
+import pytest
+
+from paper_1909_06374_gb300 import LC_FP32, LC_FP64, Plan, workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _trace(call, tmp_path):
+    path = tmp_path / "trace.json"
+    for _ in range(2):  # the first trace of a process may come without kernels
+        torch.cuda.synchronize()
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            call()
+            torch.cuda.synchronize()
+        prof.export_chrome_trace(str(path))
+        events = json.loads(path.read_text())["traceEvents"]
+        if any(e.get("cat") == "kernel" for e in events):
+            return events
+    pytest.skip("no kernel activity records on this machine")
+
+
+@pytest.mark.parametrize("prec", [LC_FP32, LC_FP64])
+@pytest.mark.parametrize("curves,log2n", [(1, 10), (1, 14), (1, 16), (8, 16), (64, 14), (1, 20)])
+def test_periodogram_of_a_few_curves_spreads_over_the_gpu(curves, log2n, prec, tmp_path):
+    """At least a block per 256 pairs of bins or two blocks per SM, whichever is fewer."""
+    with Plan([workloads.job(log2n, 0, seed=c, curve_id=c) for c in range(curves)], prec) as p:
+        x = torch.rand(p.total, dtype=p.dtype, device="cuda")
+        events = _trace(lambda: p.periodogram(x), tmp_path)
+    grids = [e["args"]["grid"][0] for e in events if e.get("cat") == "kernel" and "k_periodogram" in e["name"]]
+    assert len(grids) == 1
+    pairs = curves << (log2n - 2)
+    assert grids[0] >= min(pairs // 256, 2 * torch.cuda.get_device_properties(0).multi_processor_count)
