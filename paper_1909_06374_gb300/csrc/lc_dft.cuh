@@ -91,26 +91,33 @@ __device__ __forceinline__ void dft_regs(cplx<T> (&u)[R])
     }
 }
 
-// ---------------------------------------------------- fixed float rounding
-// The iteration ranks what the transforms return, so a float transform has to
-// round the same way in every kernel that computes it, however the compiler
-// would contract its products.  These forms write every rounding down; the
-// products that FMA leaves unrounded are the ones of the kernels' plain
-// expressions as nvcc contracts them.  FP64 transforms run one kernel per
-// length and take the plain expressions.
+// -------------------------------------------------------- fixed rounding
+// The iteration ranks what the transforms return, so a transform has to round
+// the same way in every kernel that computes it (two tile sizes, one class or
+// several per launch), however the compiler would contract its products.
+// These forms write every rounding down; the products that FMA leaves unrounded
+// are the ones of the kernels' plain expressions as nvcc contracts them.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // a b with one product of each component rounded first: a.y b.y of the real
 // part, and of the imaginary part a.y b.x (cmul_a) or a.x b.y (cmul_b).
-__device__ __forceinline__ float2 cmul_a(float2 a, float2 b)
+template <typename V> __device__ __forceinline__ V cmul_a(V a, V b)
 {
-    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+    V r;
+    r.x = fma_rn(a.x, b.x, -mul_rn(a.y, b.y));
+    r.y = fma_rn(a.x, b.y, mul_rn(a.y, b.x));
+    return r;
 }
-__device__ __forceinline__ float2 cmul_b(float2 a, float2 b)
+template <typename V> __device__ __forceinline__ V cmul_b(V a, V b)
 {
-    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+    V r;
+    r.x = fma_rn(a.x, b.x, -mul_rn(a.y, b.y));
+    r.y = fma_rn(a.y, b.x, mul_rn(a.x, b.y));
+    return r;
 }
-__device__ __forceinline__ double2 cmul_a(double2 a, double2 b) { return cmul(a, b); }
-__device__ __forceinline__ double2 cmul_b(double2 a, double2 b) { return cmul(a, b); }
 
 // a +- b as one packed operation (two float roundings, one issue slot): the
 // three transform kernels of an iteration of 4096 x 2^16 samples 1.754 -> 1.735
@@ -139,41 +146,51 @@ __device__ __forceinline__ float2 sub_fixed(float2 a, float2 b)
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
     return unpack2(r);
 }
+__device__ __forceinline__ double2 add_fixed(double2 a, double2 b)
+{
+    return make_double2(__dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y));
+}
+__device__ __forceinline__ double2 sub_fixed(double2 a, double2 b)
+{
+    return make_double2(__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y));
+}
 
 // rot16 with every rounding written down.
-template <bool INV>
-__device__ __forceinline__ float2 rot16_fixed(float2 b, int t)
+template <typename T, bool INV>
+__device__ __forceinline__ cplx<T> rot16_fixed(cplx<T> b, int t)
 {
+    cplx<T> r;
     if (t == 0) return b;
-    if (t == 4) return INV ? make_float2(-b.y, b.x) : make_float2(b.y, -b.x);
-    const float c = (float)cos16(t);
-    const float s = INV ? (float)cos16(t + 12) : -(float)cos16(t + 12);
+    if (t == 4) {
+        r.x = INV ? -b.y : b.y;
+        r.y = INV ? b.x : -b.x;
+        return r;
+    }
+    const T c = (T)cos16(t);
+    const T s = INV ? (T)cos16(t + 12) : -(T)cos16(t + 12);
     const bool x1 = t == 6 && !INV, y1 = t != 2;
-    return make_float2(x1 ? __fmaf_rn(-b.y, s, __fmul_rn(b.x, c)) : __fmaf_rn(b.x, c, -__fmul_rn(b.y, s)),
-                       y1 ? __fmaf_rn(b.y, c, __fmul_rn(b.x, s)) : __fmaf_rn(b.x, s, __fmul_rn(b.y, c)));
+    r.x = x1 ? fma_rn(-b.y, s, mul_rn(b.x, c)) : fma_rn(b.x, c, -mul_rn(b.y, s));
+    r.y = y1 ? fma_rn(b.y, c, mul_rn(b.x, s)) : fma_rn(b.x, s, mul_rn(b.y, c));
+    return r;
 }
 
 // dft_regs with every rounding written down.
 template <typename T, int R, bool INV>
 __device__ __forceinline__ void dft_fixed(cplx<T> (&u)[R])
 {
-    if constexpr (sizeof(T) == 8) {
-        dft_regs<T, R, INV>(u);
-    } else {
-        constexpr int LR = ilog2c(R);
-        BitrevSwaps<0, R, float2>::run(u);
+    constexpr int LR = ilog2c(R);
+    BitrevSwaps<0, R, cplx<T>>::run(u);
 #pragma unroll
-        for (int s = 1; s <= LR; ++s) {
-            const int m = 1 << s, h = m >> 1;
+    for (int s = 1; s <= LR; ++s) {
+        const int m = 1 << s, h = m >> 1;
 #pragma unroll
-            for (int g = 0; g < R; g += m) {
+        for (int g = 0; g < R; g += m) {
 #pragma unroll
-                for (int j = 0; j < h; ++j) {
-                    const float2 a = u[g + j];
-                    const float2 b = rot16_fixed<INV>(u[g + j + h], j * (16 / m));
-                    u[g + j] = add_fixed(a, b);
-                    u[g + j + h] = sub_fixed(a, b);
-                }
+            for (int j = 0; j < h; ++j) {
+                const cplx<T> a = u[g + j];
+                const cplx<T> b = rot16_fixed<T, INV>(u[g + j + h], j * (16 / m));
+                u[g + j] = add_fixed(a, b);
+                u[g + j + h] = sub_fixed(a, b);
             }
         }
     }

@@ -39,7 +39,7 @@ struct SmemTw {
     __device__ __forceinline__ cplx<T> operator()(uint32_t e) const
     {
         cplx<T> w = cmul_b(t1[(e >> 9) & (kTwLevel - 1)], t0[e & (kTwLevel - 1)]);
-        if (three) w = cmul(t2[e >> 18], w);
+        if (three) w = cmul_a(t2[e >> 18], w);
         return w;
     }
 };
@@ -81,8 +81,9 @@ __device__ __forceinline__ SmemTw<T> build_smem_tw(cplx<T>* mem, const cplx<T>* 
 
 // The same twiddles for the few-column tiles: W^e as the same product of the
 // same entries, read straight from the class table (a block has too few
-// elements to pay for the shared levels), and only W_R^e in shared memory.  For
-// M <= 2^18 (two levels).
+// elements to pay for the shared levels), and only W_R^e in shared memory.  FP32
+// tiles take it for M <= 2^18, where both have two levels; FP64 ones of longer
+// transforms always, the table being exact at every multiple of 2^9.
 template <typename T>
 struct DirectTw {
     const cplx<T>* rt;
@@ -200,8 +201,7 @@ __global__ void __launch_bounds__(256) k_fft_pass(const PassArgs a)
 // (rows padded to C+1 elements; each sub-pass reads its butterflies into
 // registers, then overwrites the buffer), and stores y[(i-k)R + k + q p]
 // (coalesced along i, or along q when p = 1).
-// (FP64: 16, the unit its launches are counted in; it runs kSmallCols of them
-// per block, see launch_tile_lr.)
+// (FP64: 16, as tiles of few columns have kSmallCols; see small_tiles.)
 __host__ __device__ constexpr int tile_cols(int LR, int elem_bytes)
 {
     return (LR >= 8 || elem_bytes > 8) ? 16 : (4096 >> LR);
@@ -210,15 +210,21 @@ __host__ __device__ constexpr int tile_cols(int LR, int elem_bytes)
 constexpr int kSmallCols = 4;
 constexpr int kSmallThreads = 128;
 
-template <typename T, int Q, bool INV, int LR, int C, int TH>
+// The radix-QA sub-pass of span 2^log2p2 on the tile and the radix-QB one after
+// it, in registers between the two: a butterfly of the second takes one output
+// of each of QB first ones, R/(QA QB) apart.  QA = 1: the second one alone.
+// FIRST (of span 1): the first has no twiddles, and the second's, powers of
+// W_{QA QB}, are taken without the multiplications by 1 and -+i.
+template <typename T, int QA, int QB, bool FIRST, bool INV, int LR, int C, int TH>
 __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2p2, const cplx<T>* __restrict__ tR)
 {
     using V = cplx<T>;
-    constexpr int LQ = ilog2c(Q);
+    constexpr int Q = QA * QB;
+    constexpr int LA = ilog2c(QA), LB = ilog2c(QB);
     constexpr int LC = ilog2c(C);
     constexpr int S = C + 1;                     // row stride
     constexpr int R = 1 << LR;
-    constexpr int nbq = R >> LQ;                 // butterflies per column
+    constexpr int nbq = R / Q;                   // butterflies per column
     constexpr int NB = nbq * C;                  // butterflies of the tile
     constexpr int BPT = (NB + TH - 1) / TH;      // per thread
     const int p2 = 1 << log2p2;
@@ -239,48 +245,86 @@ __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2
         if (NB % TH == 0 || b < NB) {
             const int j = b & (C - 1), i2 = b >> LC;
             const int k2 = i2 & (p2 - 1);
-            if (p2 > 1) {
-                // W_{Q p2}^{q k2} = W_R^{q k2 R/(Q p2)}, q k2 < Q p2 <= R
-                const int sh = LR - LQ - log2p2;
+            // W_{q p}^{q k} = W_R^{q k R/(q p)}, q k < q p <= R
+            auto turn = [&](V x, int e) { return INV ? cmul_b(x, cconj(tR[e])) : cmul_a(x, tR[e]); };
+            if constexpr (QA > 1) {
+                V w[QA][QB];
 #pragma unroll
-                for (int q = 1; q < Q; ++q) {
-                    const V w = tR[(q * k2) << sh];
-                    u[bi][q] = INV ? cmul_b(u[bi][q], cconj(w)) : cmul_a(u[bi][q], w);
+                for (int m = 0; m < QB; ++m) {
+                    V v[QA];
+#pragma unroll
+                    for (int q = 0; q < QA; ++q) v[q] = u[bi][m + QB * q];
+                    if (!FIRST) {
+#pragma unroll
+                        for (int q = 1; q < QA; ++q) v[q] = turn(v[q], (q * k2) << (LR - LA - log2p2));
+                    }
+                    dft_fixed<T, QA, INV>(v);
+#pragma unroll
+                    for (int q = 0; q < QA; ++q) w[q][m] = v[q];
                 }
+#pragma unroll
+                for (int q = 0; q < QA; ++q) {
+#pragma unroll
+                    for (int m = 1; m < QB; ++m) {
+                        if (!FIRST) w[q][m] = turn(w[q][m], (m * (k2 + q * p2)) << (LR - LA - LB - log2p2));
+                        else if (4 * m * q == Q) w[q][m] = rot16_fixed<T, INV>(w[q][m], 4);
+                        else if (q) w[q][m] = turn(w[q][m], (m * q) << (LR - LA - LB));
+                    }
+                    dft_fixed<T, QB, INV>(w[q]);
+#pragma unroll
+                    for (int m = 0; m < QB; ++m) u[bi][m * QA + q] = w[q][m];
+                }
+            } else {
+                if (!FIRST) {
+#pragma unroll
+                    for (int q = 1; q < QB; ++q) u[bi][q] = turn(u[bi][q], (q * k2) << (LR - LB - log2p2));
+                }
+                dft_fixed<T, QB, INV>(u[bi]);
             }
-            dft_fixed<T, Q, INV>(u[bi]);
-            const int jo = ((i2 - k2) << LQ) + k2;
+            const int jo = (i2 - k2) * Q + k2;
 #pragma unroll
             for (int q = 0; q < Q; ++q) buf[(jo + q * p2) * S + j] = u[bi][q];
         }
     }
 }
 
-// All radix-2^LR sub-passes of one tile of C columns, in place in `buf`: a
-// radix-2/4/8 sub-pass for LR mod 4, then radix-16 ones.  Ends with a block
-// barrier.
+// All sub-passes of a radix-2^LR pass on one tile of C columns, in place in
+// `buf`.  FP32: a radix-2/4/8 one for LR mod 4, then radix-16 ones.  FP64: a
+// radix-2 one for odd LR, then radix-4 ones, which give four times the threads
+// work in the tiles of few columns (a warp's FP64 operation holds its
+// scheduler's FP64 unit for 64 clocks, so few warps with long butterflies leave
+// most of it idle).  Full FP64 tiles, which fill the GPU, take the radix-4 ones
+// in pairs (from 2^7 on, where the threads have enough of them): the same
+// operations less the first pair's trivial twiddles, 24 per point in place of
+// 25 at 2^8 and 21 of 23 at 2^7 (transforms of 512 curves of 2^16 4.87 -> 4.67
+// ms per iteration, of 2^15 2.40 -> 2.26).  Ends with a block barrier.
 template <typename T, bool INV, int LR, int C, int TH>
 __device__ __forceinline__ void tile_dft(cplx<T>* __restrict__ buf, const cplx<T>* __restrict__ tR)
 {
-    // FP64 tiles of few columns: radix-4 sub-passes, four times the threads at
-    // work (a warp's FP64 operation holds its scheduler's FP64 unit for 64
-    // clocks, so few warps with long butterflies leave most of it idle)
-    constexpr int LQ = sizeof(T) == 8 && C == kSmallCols ? 2 : 4;
-    constexpr int rem = LR % LQ;
+    constexpr int LQ = sizeof(T) == 8 ? 2 : 4;
+    constexpr int L0 = LR % LQ ? LR % LQ : LQ;  // the first sub-pass
+    constexpr bool PAIRS = sizeof(T) == 8 && C > kSmallCols && LR >= 7;
     int log2p2 = 0;
-    if (rem) {
-        tile_subpass<T, (1 << (rem ? rem : 1)), INV, LR, C, TH>(buf, 0, tR);
+    if constexpr (PAIRS) {
+        tile_subpass<T, (1 << L0), 4, true, INV, LR, C, TH>(buf, 0, tR);
+        log2p2 = L0 + 2;
         __syncthreads();
-        log2p2 = rem;
+        for (; log2p2 + 4 <= LR; log2p2 += 4) {
+            tile_subpass<T, 4, 4, false, INV, LR, C, TH>(buf, log2p2, tR);
+            __syncthreads();
+        }
+    } else {
+        tile_subpass<T, 1, (1 << L0), true, INV, LR, C, TH>(buf, 0, tR);
+        log2p2 = L0;
+        __syncthreads();
     }
     for (; log2p2 < LR; log2p2 += LQ) {
-        tile_subpass<T, (1 << LQ), INV, LR, C, TH>(buf, log2p2, tR);
+        tile_subpass<T, 1, (1 << LQ), false, INV, LR, C, TH>(buf, log2p2, tR);
         __syncthreads();
     }
 }
 
-// SMALL: tiles of kSmallCols columns on kSmallThreads threads, for transforms
-// whose full tiles would leave most of the GPU idle (launch_tile_set).
+// SMALL: tiles of kSmallCols columns on kSmallThreads threads (small_tiles).
 template <typename T, int LR, bool INV, bool MULTI, bool SMALL>
 __global__ void __launch_bounds__(SMALL ? kSmallThreads : 256, SMALL ? 4 : (sizeof(T) == 4 && LR < 9) ? 4 : 2)
     k_fft_tile(const __grid_constant__ LaunchSet<PassArgs> set)
@@ -327,7 +371,7 @@ __global__ void __launch_bounds__(SMALL ? kSmallThreads : 256, SMALL ? 4 : (size
             const uint32_t k = (i0 + (uint32_t)j) & (p - 1);
             V w = tw(((uint32_t)r * k) << (a.log2M - LR - a.log2p));
             if (INV) w.y = -w.y;
-            x = cmul_b(x, w);
+            x = sizeof(T) == 8 && !INV ? cmul_a(x, w) : cmul_b(x, w);
         }
         b0[r * S + j] = x;
     }
@@ -489,8 +533,7 @@ __global__ void __launch_bounds__(256) k_spectral_tk(const SpecArgs a)
     }
 }
 
-// keep_phase and pack_pair of the tile path, every float rounding written down
-// (lc_dft.cuh).
+// keep_phase of the tile path, every rounding written down (lc_dft.cuh).
 __device__ __forceinline__ float2 keep_phase_fixed(float2 X, float A)
 {
     const float m2 = __fmaf_rn(X.x, X.x, __fmul_rn(X.y, X.y));
@@ -498,7 +541,13 @@ __device__ __forceinline__ float2 keep_phase_fixed(float2 X, float A)
     const float s = __fmul_rn(A, rsqrtf(m2));
     return make_float2(__fmul_rn(X.x, s), __fmul_rn(X.y, s));
 }
-__device__ __forceinline__ double2 keep_phase_fixed(double2 X, double A) { return keep_phase(X, A); }
+__device__ __forceinline__ double2 keep_phase_fixed(double2 X, double A)
+{
+    const double m2 = __fma_rn(X.x, X.x, __dmul_rn(X.y, X.y));
+    if (m2 == 0.0) return make_double2(A, 0.0);
+    const double s = __ddiv_rn(A, __dsqrt_rn(m2));
+    return make_double2(__dmul_rn(X.x, s), __dmul_rn(X.y, s));
+}
 
 // One conjugate pair (t, M - t) of the spectral step on values held by the
 // caller: za = Z_t, zb = Z_{M-t} in, Z'_t, Z'_{M-t} out.  The arithmetic runs
@@ -774,10 +823,8 @@ static cudaError_t tile_attrs()
     const int small = (int)tile_smem_bytes<T>(LR, kTileMaxLog2M, true);
     cudaError_t e = tile_attrs_m<T, LR, false, true>(small);
     if (e == cudaSuccess) e = tile_attrs_m<T, LR, true, true>(small);
-    if constexpr (sizeof(T) == 4) {
-        if (e == cudaSuccess) e = tile_attrs_m<T, LR, false, false>(smem);
-        if (e == cudaSuccess) e = tile_attrs_m<T, LR, true, false>(smem);
-    }
+    if (e == cudaSuccess) e = tile_attrs_m<T, LR, false, false>(smem);
+    if (e == cudaSuccess) e = tile_attrs_m<T, LR, true, false>(smem);
     return e;
 }
 
@@ -802,19 +849,21 @@ cudaError_t fft_kernel_attributes()
 }
 
 // Whether a launch of `blocks` full tiles takes tiles of kSmallCols columns
-// instead: where the full tiles (four or two resident per SM) give fewer than
-// two blocks per SM, the time is one block's, and a block of a quarter of the
-// columns or less is done sooner: one 2^17 curve's three transform kernels 20.5
-// -> 14.9 us per iteration.  FP64 transforms, bound by the FP64 rate, always
-// take them, with radix-4 sub-passes: one FP64 2^14 curve 78 -> 30 us per
-// iteration, and a curve's rounding does not depend on its batch; float tiles
-// round alike in both sizes.
-static bool small_tiles(const LaunchSet<PassArgs>& s, uint32_t blocks)
+// instead (both round alike).  FP32: where the full tiles (four or two resident
+// per SM) give fewer than two blocks per SM, the time is one block's, and a
+// block of a quarter of the columns or less is done sooner: one 2^17 curve's
+// three transform kernels 20.5 -> 14.9 us per iteration.  FP64, bound by the
+// FP64 rate with two full tiles resident per SM: below three waves of them,
+// where small ones leave less of the last one empty (us of four iterations,
+// small/full: 64 curves of 2^16 3880/4010, 128 7403/7351, 512 28320/27500;
+// one 2^14 curve 306/484), and in the spectral kernel of radices below 2^7,
+// whose full tiles have too few butterflies for their threads (1216 curves of
+// 2^13 5549/5745).
+static bool small_tiles(const LaunchSet<PassArgs>& s, uint32_t blocks, bool fp64)
 {
-    if (blocks >= 152 * 2) return false;
     for (int i = 0; i < s.n; ++i)
-        if (s.c[i].log2M > 18) return false;  // the full tiles' twiddles have a third level there
-    return true;
+        if (s.c[i].log2M > 18) return fp64;  // the full tiles' twiddles have a third level there
+    return blocks < 152u * 2u * (fp64 ? 3u : 1u);
 }
 
 // The launch set with every entry's blocks times f (full tiles to small ones).
@@ -830,13 +879,13 @@ static LaunchSet<PassArgs> scaled_set(const LaunchSet<PassArgs>& s, uint32_t f)
 template <typename T, int LR, bool INV>
 static void launch_tile_lr(const LaunchSet<PassArgs>& s, uint32_t blocks, size_t smem, bool multi, cudaStream_t st)
 {
-    if (sizeof(T) == 8 || small_tiles(s, blocks)) {
+    if (small_tiles(s, blocks, sizeof(T) == 8)) {
         constexpr uint32_t f = tile_cols(LR, (int)sizeof(cplx<T>)) / kSmallCols;
         const LaunchSet<PassArgs> r = scaled_set(s, f);
         smem = tile_smem_bytes<T>(LR, 0, true);
         if (multi) k_fft_tile<T, LR, INV, true, true><<<blocks * f, kSmallThreads, smem, st>>>(r);
         else k_fft_tile<T, LR, INV, false, true><<<blocks * f, kSmallThreads, smem, st>>>(r);
-    } else if constexpr (sizeof(T) == 4) {
+    } else {
         if (multi) k_fft_tile<T, LR, INV, true, false><<<blocks, 256, smem, st>>>(s);
         else k_fft_tile<T, LR, INV, false, false><<<blocks, 256, smem, st>>>(s);
     }
@@ -846,13 +895,13 @@ template <typename T, int LR>
 static void launch_spectral_lr(const LaunchSet<PassArgs>& s, uint32_t blocks, size_t smem, bool multi, const void* A,
                                cudaStream_t st)
 {
-    if (sizeof(T) == 8 || small_tiles(s, blocks)) {
+    if (small_tiles(s, blocks, sizeof(T) == 8) || (sizeof(T) == 8 && LR < 7)) {
         constexpr uint32_t f = tile_cols(LR, (int)sizeof(cplx<T>)) / kSmallCols;
         const LaunchSet<PassArgs> r = scaled_set(s, f);
         smem = tile_smem_bytes<T>(LR, 0, true);
         if (multi) k_fft_spectral<T, LR, true, true><<<blocks * f, kSmallThreads, smem, st>>>(r, A);
         else k_fft_spectral<T, LR, false, true><<<blocks * f, kSmallThreads, smem, st>>>(r, A);
-    } else if constexpr (sizeof(T) == 4) {
+    } else {
         if (multi) k_fft_spectral<T, LR, true, false><<<blocks, 256, smem, st>>>(s, A);
         else k_fft_spectral<T, LR, false, false><<<blocks, 256, smem, st>>>(s, A);
     }
