@@ -27,7 +27,10 @@ constexpr int kSpecTile = kSpecBlock * kSpecPerThread;  // bins per block
 // terms); the amplitude sqrt(P/2) sqrt(-2 ln U1) as one square root: these are
 // the FP64 operations that the FP64-rate-bound kernels spend their time on
 // (conversions of 64-bit integers are among them: the uniforms, 2 U2 and j are
-// put together from their bits, with one exact subtraction each at most).
+// put together from their bits, with one exact subtraction each at most).  Two
+// kernels compute the coefficients and two add their squares, by the number of
+// a class's curves, so every operation that nvcc could contract with another is
+// written down: a curve's amplitudes do not depend on its batch.
 __device__ __forceinline__ double2 tk_bin(const CurveDev& cv, double c, bool fixed, uint64_t j, uint64_t nh, double& P)
 {
     const uint4 w = philox(j, cv.curve_id, 0u, cv.seed);
@@ -36,13 +39,21 @@ __device__ __forceinline__ double2 tk_bin(const CurveDev& cv, double c, bool fix
     double sn, cs;
     sincospi(__hiloint2double(__double2hiint(U2) + 0x100000, __double2loint(U2)), &sn, &cs);  // 2 U2, by its exponent
     // j as a double: the low word of 2^52 + j, less 2^52 (j < 2^32, exact)
-    const double ly = log((__hiloint2double(0x43300000, (int)(uint32_t)j) - 0x1p52) * c);
-    P = 1.0 / (exp(cv.a_lo * ly) + exp(cv.a_hi * ly));
+    const double ly = log(__dmul_rn(__dsub_rn(__hiloint2double(0x43300000, (int)(uint32_t)j), 0x1p52), c));
+    P = __ddiv_rn(1.0, __dadd_rn(exp(__dmul_rn(cv.a_lo, ly)), exp(__dmul_rn(cv.a_hi, ly))));
     if (j < nh) {
-        const double a = fixed ? sqrt(P) : sqrt(-P * lu);
-        return make_double2(a * cs, a * sn);
+        const double a = fixed ? __dsqrt_rn(P) : __dsqrt_rn(__dmul_rn(-P, lu));
+        return make_double2(__dmul_rn(a, cs), __dmul_rn(a, sn));
     }
-    return make_double2(fixed ? (cs < 0.0 ? -sqrt(P) : sqrt(P)) : sqrt(-2.0 * P * lu) * cs, 0.0);
+    const double a = fixed ? __dsqrt_rn(P) : __dsqrt_rn(__dmul_rn(__dmul_rn(-2.0, P), lu));
+    return make_double2(fixed ? (cs < 0.0 ? -a : a) : __dmul_rn(a, cs), 0.0);
+}
+
+// acc + the share of coefficient j in the series' variance.
+__device__ __forceinline__ double tk_add_power(double acc, double2 X, uint64_t j, uint64_t nh)
+{
+    if (j < nh) return __fma_rn(2.0, __fma_rn(X.x, X.x, __dmul_rn(X.y, X.y)), acc);
+    return __fma_rn(X.x, X.x, acc);
 }
 
 // Tree sums of the block's kSpecBlock values (fixed order), in thread 0.
@@ -60,7 +71,8 @@ __device__ __forceinline__ void spec_block_sums(double (&red)[kSpecBlock], doubl
 
 __global__ void __launch_bounds__(kSpecBlock)
 k_tk_spectrum(const CurveDev* __restrict__ curves, const int* __restrict__ cls_curves,
-              int blocks_per_curve, double2* __restrict__ spec, double* __restrict__ partial, double* __restrict__ partial_p)
+              int blocks_per_curve, double2* __restrict__ spec, double* __restrict__ partial,
+              double* __restrict__ partial_p)
 {
     const int ci = blockIdx.x / blocks_per_curve;
     const int jb = blockIdx.x % blocks_per_curve;
@@ -77,13 +89,8 @@ k_tk_spectrum(const CurveDev* __restrict__ curves, const int* __restrict__ cls_c
         if (j > 0) {
             double P;
             X = tk_bin(cv, c, fixed, j, nh, P);
-            if (j < nh) {
-                acc += 2.0 * (X.x * X.x + X.y * X.y);
-                acc_p += 2.0 * P;
-            } else {
-                acc += X.x * X.x;
-                acc_p += P;
-            }
+            acc = tk_add_power(acc, X, j, nh);
+            acc_p += j < nh ? 2.0 * P : P;
         }
         spec[cv.offh + j] = X;
     }
@@ -120,7 +127,8 @@ __global__ void __launch_bounds__(kFewBins) k_tk_bins(const CurveDev* __restrict
 
 __global__ void __launch_bounds__(kSpecBlock) k_tk_sums(const CurveDev* __restrict__ curves,
                                                         const int* __restrict__ cls_curves, int blocks_per_curve,
-                                                        const double2* __restrict__ spec, double* __restrict__ partial, double* __restrict__ partial_p)
+                                                        const double2* __restrict__ spec,
+                                                        double* __restrict__ partial, double* __restrict__ partial_p)
 {
     const int jb = blockIdx.x % blocks_per_curve;
     const CurveDev& cv = curves[cls_curves[blockIdx.x / blocks_per_curve]];
@@ -136,8 +144,7 @@ __global__ void __launch_bounds__(kSpecBlock) k_tk_sums(const CurveDev* __restri
     for (int q = 0; q < kSpecPerThread; ++q) {
         const uint64_t j = (uint64_t)jb * kSpecTile + (uint64_t)q * kSpecBlock + threadIdx.x;
         if (j > nh || j == 0) continue;
-        if (j < nh) acc += 2.0 * (X[q].x * X[q].x + X[q].y * X[q].y);
-        else acc += X[q].x * X[q].x;
+        acc = tk_add_power(acc, X[q], j, nh);
     }
     __shared__ double red[kSpecBlock], red_p[kSpecBlock];
     red[threadIdx.x] = acc;
@@ -152,9 +159,10 @@ __global__ void __launch_bounds__(kSpecBlock) k_tk_sums(const CurveDev* __restri
 // sigma (realised) and sigma_P (PSD) of each curve of a class: the partial
 // sums added in block order.
 constexpr int kSigmaWarps = 4;
-__global__ void __launch_bounds__(32 * kSigmaWarps) k_sigma(const int* __restrict__ cls_curves, int ncurves, int blocks_per_curve,
-                        const double* __restrict__ partial, const double* __restrict__ partial_p,
-                        double* __restrict__ sigma, double* __restrict__ sigma_p)
+__global__ void __launch_bounds__(32 * kSigmaWarps) k_sigma(const int* __restrict__ cls_curves, int ncurves,
+                                                            int blocks_per_curve, const double* __restrict__ partial,
+                                                            const double* __restrict__ partial_p,
+                                                            double* __restrict__ sigma, double* __restrict__ sigma_p)
 {
     // one warp per curve: 32 partials of each sum are loaded at once, then lane
     // 0 adds one sum and lane 1 the other (one thread per curve loading and
@@ -408,8 +416,8 @@ int launch_tk_spectrum(const Plan& p, const ClassInfo& k, cudaStream_t st)
     } else {
         k_tk_spectrum<<<k.ncurves * bpc, kSpecBlock, 0, st>>>(p.d_curves, k.d_curves, bpc, p.d_spec, part, part_p);
     }
-    k_sigma<<<(k.ncurves + kSigmaWarps - 1) / kSigmaWarps, 32 * kSigmaWarps, 0, st>>>(k.d_curves, k.ncurves, bpc, part, part_p, p.d_sigma,
-                                                     p.d_sigma + p.ncurves);
+    k_sigma<<<(k.ncurves + kSigmaWarps - 1) / kSigmaWarps, 32 * kSigmaWarps, 0, st>>>(
+        k.d_curves, k.ncurves, bpc, part, part_p, p.d_sigma, p.d_sigma + p.ncurves);
     return few ? 3 : 2;
 }
 
