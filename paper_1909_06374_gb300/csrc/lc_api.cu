@@ -592,7 +592,10 @@ static lc_status run_iterations_impl(Plan& p, uint32_t override_iters, uint32_t 
             return LC_OK;
         };
         uint32_t it = 0;
-        if (p.total <= kGraphSamples && n_it >= 2 * kGraphIters) {
+        bool radix = false;
+        for (auto& k : p.classes) radix |= !k.resident && !k.bucket && !k.rank_cta;
+        const bool repaid = p.replayed + std::max(n_it, p.max_iters) >= (radix ? kGraphRepayRadix : kGraphRepay);
+        if (p.total <= kGraphSamples && n_it >= 2 * kGraphIters && (p.iter_graphs || repaid)) {
             const lc_status gs = instantiate(p.iter_graphs, kGraphIters);
             if (gs != LC_OK) return gs;
             for (; it + kGraphIters <= n_it; it += kGraphIters) LC_CK(cudaGraphLaunch(p.iter_graphs, st));
@@ -602,6 +605,7 @@ static lc_status run_iterations_impl(Plan& p, uint32_t override_iters, uint32_t 
             if (gs != LC_OK) return gs;
         }
         for (; it < n_it; ++it) LC_CK(cudaGraphLaunch(p.iter_graph, st));
+        p.replayed += n_it;
         *launches += (uint64_t)n_it * p.launches_per_iter;
     } else if (n_it > 0) {
         launch_iter_add(p, n_it, st);

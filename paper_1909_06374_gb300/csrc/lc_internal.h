@@ -85,6 +85,7 @@ struct Plan {
     bool timed_setup = false, timed_iter = false;
     cudaGraphExec_t iter_graph = nullptr;   // one iteration
     cudaGraphExec_t iter_graphs = nullptr;  // kGraphIters of them (small plans)
+    uint64_t replayed = 0;                  // iterations run from either
     uint64_t launches_per_iter = 0;
     uint64_t last_launches = 0;
     bool setup_done = false;
@@ -103,8 +104,16 @@ struct Plan {
 // Iterations per graph of a small plan (at most kGraphSamples samples): the gap
 // between two graphs of a stream is about 3 us, of the 49 us that an iteration
 // of one 2^17 curve takes; larger plans have nothing to gain for the longer
-// instantiation.
+// instantiation.  That costs the host about 2 us per kernel more than a graph of
+// one iteration, so it is made for a plan with kGraphRepay iterations behind or
+// before it (kGraphRepayRadix where radix passes put 20 to 30 kernels in an
+// iteration).  A new plan's first 8 iterations with graphs of one / of four: one
+// FP32 curve of 2^8 517 / 620 us, of 2^13 456 / 489, FP64 2^9 1107 / 1263; first
+// 20: 2^13 906 / 914, 2^17 1290 / 1264, FP64 2^13 1049 / 1011; first 100: 2^8
+// 4664 / 4612, FP64 2^9 11197 / 11158.
 constexpr uint32_t kGraphIters = 4;
+constexpr uint64_t kGraphRepay = 20;
+constexpr uint64_t kGraphRepayRadix = 96;
 constexpr size_t kGraphSamples = (size_t)1 << 20;
 
 // CUDA events around the kernel groups of one profiled iteration.

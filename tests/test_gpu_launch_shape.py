@@ -9,15 +9,19 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-def _trace(call, tmp_path):
+def _trace_once(call, tmp_path):
     path = tmp_path / "trace.json"
-    for _ in range(2):  # the first trace of a process may come without kernels
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
         torch.cuda.synchronize()
-        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-            call()
-            torch.cuda.synchronize()
-        prof.export_chrome_trace(str(path))
-        events = json.loads(path.read_text())["traceEvents"]
+    prof.export_chrome_trace(str(path))
+    return json.loads(path.read_text())["traceEvents"]
+
+
+def _trace(call, tmp_path):
+    for _ in range(2):  # the first trace of a process may come without kernels
+        events = _trace_once(call, tmp_path)
         if any(e.get("cat") == "kernel" for e in events):
             return events
     pytest.skip("no kernel activity records on this machine")
@@ -45,3 +49,21 @@ def test_fp64_batches_take_full_tiles(curves, log2n, threads, tmp_path):
         events = _trace(lambda: p.periodogram(x), tmp_path)
     blocks = {e["args"]["block"][0] for e in events if e.get("cat") == "kernel" and "k_fft_tile" in e["name"]}
     assert blocks == {threads}
+
+
+@pytest.mark.parametrize("log2n,iters,calls,graphs", [(13, 8, 4, [8, 8, 2, 2]), (13, 10, 2, [10, 4]),
+                                                      (13, 34, 2, [10, 10]), (8, 34, 3, [34, 34, 10]),
+                                                      (8, 100, 1, [25])])
+def test_graphs_of_several_iterations_where_they_repay(log2n, iters, calls, graphs, tmp_path):
+    """A plan of few iterations replays a graph of one: the longer graph's
+    instantiation costs more than it saves until enough have been run."""
+    with Plan([workloads.job(log2n, iters, seed=3, curve_id=0)], LC_FP32) as warm:
+        _trace(warm.generate, tmp_path)
+    with Plan([workloads.job(log2n, iters, seed=3, curve_id=0)], LC_FP32) as p:
+        p.setup()
+        x = p.get_state()
+        for want in graphs[:calls]:
+            events = _trace_once(lambda: p.iterate(iters), tmp_path)
+            got = sum(e.get("name", "").startswith("cudaGraphLaunch") for e in events)
+            assert got == want
+            p.set_state(x)
