@@ -109,38 +109,37 @@ __global__ void __launch_bounds__(256) k_periodogram(const int* __restrict__ cls
 // that walks the whole curve, two loads per pair and nothing kept: 3.14 ms.
 constexpr int kSfBatch = 16;  // lags whose runs are added up together
 
-// Sum of 256 runs (>= 0, or NaN), 16 by each of 16 neighbouring threads: r[0],
-// r[16], ... of the thread's r; 0 where !on.  In the first of the 16 threads.
-// Added as integers, 2^-54 of the largest run's power of two as unit: exact for
-// the runs above 2^-31 of it, and below 2^-46 of the sum in all (255 FP64
-// additions: 2^-45), over the whole range of float.  256 curves of 2^16 samples
-// at 53 lags 231 us, with FP64 additions (16 clocks per warp operation) 251;
-// 2000 curves of 2^10 at 27 lags 51 against 95.  Infinities and NaN go there.
-__device__ __forceinline__ double sum_runs(const float* r, bool on)
+// Sum of the 256 runs at r (>= 0, or NaN) by a warp, in lane 0.  Added as
+// integers, 2^-54 of the largest run's power of two as unit: exact for the runs
+// above 2^-31 of it, and below 2^-46 of the sum in all (255 FP64 additions:
+// 2^-45), over the whole range of float.  256 curves of 2^16 samples at 53 lags
+// 233 us, with FP64 additions (16 clocks per warp operation) 258; 2000 curves of
+// 2^10 at 27 lags 62 against 117.  Infinities and NaN go there.
+__device__ __forceinline__ double sum_runs(const float* r)
 {
+    const int lane = threadIdx.x & 31;
     uint32_t top = 0u;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) top = max(top, on ? __float_as_uint(r[16 * q]) : 0u);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-    if (__any_sync(0xffffffffu, top >= 0x7f800000u)) {
+    for (int q = 0; q < 8; ++q) top = max(top, __float_as_uint(r[lane + 32 * q]));
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (top >= 0x7f800000u) {
         double sum = 0.0;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) sum += on ? (double)r[16 * q] : 0.0;
+        for (int q = 0; q < 8; ++q) sum += (double)r[lane + 32 * q];
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o, 16);
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
         return sum;
     }
     const uint32_t et = max(top >> 23, 1u);
     unsigned long long acc = 0u;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const uint32_t v = on ? __float_as_uint(r[16 * q]) : 0u, e = v >> 23;
+    for (int q = 0; q < 8; ++q) {
+        const uint32_t v = __float_as_uint(r[lane + 32 * q]), e = v >> 23;
         const uint32_t m = e ? (v & 0x7fffffu) | 0x800000u : v;
         acc += ((unsigned long long)m << 31) >> min(et - max(e, 1u), 63u);
     }
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o, 16);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     return (double)acc * __hiloint2double((int)((1023u + et - 181u) << 20), 0);
 }
 
@@ -150,7 +149,7 @@ __global__ void __launch_bounds__(256, 2)
                      int groups, int per, int nlags, const uint32_t* __restrict__ lags, const float* __restrict__ x,
                      double* __restrict__ part, double* __restrict__ out)
 {
-    __shared__ float sh[kSfBatch][256 + 16];  // rows half a bank cycle apart
+    __shared__ float sh[kSfBatch][256];
     const int t = threadIdx.x;
     const int g = (int)(blockIdx.x % (uint32_t)groups);
     const int seg = (int)((blockIdx.x / (uint32_t)groups) % (uint32_t)segs);
@@ -186,11 +185,12 @@ __global__ void __launch_bounds__(256, 2)
             sh[b][t] = run;
         }
         __syncthreads();
-        const int b = t >> 4;
-        const double sum = sum_runs(&sh[b][t & 15], b < nb);
-        if (b < nb && (t & 15) == 0) {
-            if (segs == 1) out[(size_t)c * nlags + lb + b] = sum / (double)(n - lags[lb + b]);
-            else part[off / 2 + (size_t)(lb + b) * segs + seg] = sum;
+        for (int b = t >> 5; b < nb; b += 8) {
+            const double sum = sum_runs(sh[b]);
+            if ((t & 31) == 0) {
+                if (segs == 1) out[(size_t)c * nlags + lb + b] = sum / (double)(n - lags[lb + b]);
+                else part[off / 2 + (size_t)(lb + b) * segs + seg] = sum;
+            }
         }
         __syncthreads();
     }
