@@ -849,21 +849,23 @@ cudaError_t fft_kernel_attributes()
 }
 
 // Whether a launch of `blocks` full tiles takes tiles of kSmallCols columns
-// instead (both round alike).  FP32: where the full tiles (four or two resident
-// per SM) give fewer than two blocks per SM, the time is one block's, and a
-// block of a quarter of the columns or less is done sooner: one 2^17 curve's
-// three transform kernels 20.5 -> 14.9 us per iteration.  FP64, bound by the
-// FP64 rate with two full tiles resident per SM: below three waves of them,
-// where small ones leave less of the last one empty (us of four iterations,
-// small/full: 64 curves of 2^16 3880/4010, 128 7403/7351, 512 28320/27500;
-// one 2^14 curve 306/484), and in the spectral kernel of radices below 2^7,
-// whose full tiles have too few butterflies for their threads (1216 curves of
-// 2^13 5549/5745).
+// instead (both round alike).  FP32: below half a full tile per SM, where the
+// time is one block's and a block of a quarter of the columns or less is done
+// sooner; with more of them the small tiles' narrow rows and twiddle reads cost
+// more (us of an iteration's three transform kernels, small/full: one 2^13
+// curve 9.8/17.9, 76 of them 19.4/17.4, 280 47.6/23.8; 8, 14 and 36 curves of
+// 2^16 16.8/19.8, 23.1/19.6, 47.7/25.2; 2, 3 and 5 of 2^19 29.0/37.3, 37.2/38.2,
+// 56.7/51.2).  FP64, bound by the FP64 rate with two full tiles resident per SM:
+// below three waves of them, where small ones leave less of the last one empty
+// (us of four iterations, small/full: 64 curves of 2^16 3880/4010, 128
+// 7403/7351, 512 28320/27500; one 2^14 curve 306/484), and in the spectral
+// kernel of radices below 2^7, whose full tiles have too few butterflies for
+// their threads (1216 curves of 2^13 5549/5745).
 static bool small_tiles(const LaunchSet<PassArgs>& s, uint32_t blocks, bool fp64)
 {
     for (int i = 0; i < s.n; ++i)
         if (s.c[i].log2M > 18) return fp64;  // the full tiles' twiddles have a third level there
-    return blocks < 152u * 2u * (fp64 ? 3u : 1u);
+    return fp64 ? blocks < 152 * 2 * 3 : blocks < 152 / 2;
 }
 
 // The launch set with every entry's blocks times f (full tiles to small ones).

@@ -40,11 +40,14 @@ def test_periodogram_of_a_few_curves_spreads_over_the_gpu(curves, log2n, prec, t
     assert grids[0] >= min(pairs // 256, 2 * torch.cuda.get_device_properties(0).multi_processor_count)
 
 
-@pytest.mark.parametrize("curves,log2n,threads", [(1, 16, 128), (128, 16, 256), (16, 18, 256)])
-def test_fp64_batches_take_full_tiles(curves, log2n, threads, tmp_path):
-    """Tiles of few columns (128 threads) for a few curves only: batches are
-    bound by the FP64 rate, and full tiles spend fewer operations per point."""
-    with Plan([workloads.job(log2n, 0, seed=c, curve_id=c) for c in range(curves)], LC_FP64) as p:
+@pytest.mark.parametrize("prec,curves,log2n,threads", [(LC_FP64, 1, 16, 128), (LC_FP64, 128, 16, 256),
+                                                       (LC_FP64, 16, 18, 256), (LC_FP32, 1, 16, 128),
+                                                       (LC_FP32, 8, 17, 256), (LC_FP32, 200, 13, 256),
+                                                       (LC_FP32, 4, 19, 256)])
+def test_batches_take_full_tiles(prec, curves, log2n, threads, tmp_path):
+    """Tiles of few columns (128 threads) where full ones would leave most of
+    the GPU idle, and only there."""
+    with Plan([workloads.job(log2n, 0, seed=c, curve_id=c) for c in range(curves)], prec) as p:
         x = torch.rand(p.total, dtype=p.dtype, device="cuda")
         events = _trace(lambda: p.periodogram(x), tmp_path)
     blocks = {e["args"]["block"][0] for e in events if e.get("cat") == "kernel" and "k_fft_tile" in e["name"]}
