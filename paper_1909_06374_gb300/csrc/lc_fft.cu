@@ -39,7 +39,8 @@ struct SmemTw {
     __device__ __forceinline__ cplx<T> operator()(uint32_t e) const
     {
         cplx<T> w = cmul_b(t1[(e >> 9) & (kTwLevel - 1)], t0[e & (kTwLevel - 1)]);
-        if (three) w = cmul_a(t2[e >> 18], w);
+        // (FP64 tiles of three levels take DirectTw; a branch here costs its operations untaken)
+        if (sizeof(T) == 4 && three) w = cmul_a(t2[e >> 18], w);
         return w;
     }
 };
@@ -296,8 +297,8 @@ __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2
 // most of it idle).  Full FP64 tiles, which fill the GPU, take the radix-4 ones
 // in pairs (from 2^7 on, where the threads have enough of them): the same
 // operations less the first pair's trivial twiddles, 24 per point in place of
-// 25 at 2^8 and 21 of 23 at 2^7 (transforms of 512 curves of 2^16 4.87 -> 4.67
-// ms per iteration, of 2^15 2.40 -> 2.26).  Ends with a block barrier.
+// 25 at 2^8 and 21 of 23 at 2^7 (four iterations of 512 curves of 2^16 27.8 ->
+// 26.9 ms).  Ends with a block barrier.
 template <typename T, bool INV, int LR, int C, int TH>
 __device__ __forceinline__ void tile_dft(cplx<T>* __restrict__ buf, const cplx<T>* __restrict__ tR)
 {
@@ -379,7 +380,7 @@ __global__ void __launch_bounds__(SMALL ? kSmallThreads : 256, SMALL ? 4 : (size
     tile_dft<T, INV, LR, C, TH>(b0, tw.tR);
     const V* in = b0;
     const uint32_t smask = (1u << a.smp_shift) - 1u, shalf = (smask + 1u) >> 1;
-    float* const smp = INV && a.smp ? a.smp + (size_t)ci * a.smp_words : nullptr;
+    float* const smp = INV && sizeof(T) == 4 && a.smp ? a.smp + (size_t)ci * a.smp_words : nullptr;
     if (p >= (uint32_t)C) {
         for (int idx = threadIdx.x; idx < R * C; idx += TH) {
             const int q = idx >> LC, j = idx & (C - 1);
@@ -857,10 +858,10 @@ cudaError_t fft_kernel_attributes()
 // 2^16 16.8/19.8, 23.1/19.6, 47.7/25.2; 2, 3 and 5 of 2^19 29.0/37.3, 37.2/38.2,
 // 56.7/51.2).  FP64, bound by the FP64 rate with two full tiles resident per SM:
 // below three waves of them, where small ones leave less of the last one empty
-// (us of four iterations, small/full: 64 curves of 2^16 3880/4010, 128
-// 7403/7351, 512 28320/27500; one 2^14 curve 306/484), and in the spectral
-// kernel of radices below 2^7, whose full tiles have too few butterflies for
-// their threads (1216 curves of 2^13 5549/5745).
+// (us of four iterations, small/full: 48 curves of 2^16 3064/3189, 96 5683/5746,
+// 128 7312/7202; one 2^14 curve 306/480), and in the spectral kernel of radices
+// below 2^7, whose full tiles have too few butterflies for their threads (1216
+// curves of 2^13 5518/5720).
 static bool small_tiles(const LaunchSet<PassArgs>& s, uint32_t blocks, bool fp64)
 {
     for (int i = 0; i < s.n; ++i)
