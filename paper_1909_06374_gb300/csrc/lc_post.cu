@@ -19,13 +19,15 @@ namespace lc {
 // E = (Z_k + conj Z_{M-k})/2, O = (Z_k - conj Z_{M-k})/(2i).
 // P_j = |X_j|^2 2/N^2 (Eq. A2) or |X_j|^2 2 dt N / X_0^2 (Eq. A4, X_0 = N mu).
 //
-// One block takes `pairs` conjugate pairs of one curve (launch_periodogram).  A float bin's
-// power takes two FP64 operations (three for Eq. A4) of the 2 per clock and SM:
-// its conversions and Eq. A2's scale, a power of two, are put together from
-// bits.  2048 curves of 2^16 samples, transform included: 1.11 ms with FP64
-// conversions and scaling (Eq. A4, with a division per bin: 1.81), 0.976 (1.03)
-// with these.
-constexpr uint32_t kPgPairs = 4096;
+// One block takes `pairs` conjugate pairs of one curve (launch_periodogram).  A
+// float bin's power takes two FP64 operations (three for Eq. A4) of the 2 per
+// clock and SM: its conversions and Eq. A2's scale, a power of two, are put
+// together from bits.  2048 curves of 2^16 samples, transform included: 1.11 ms with FP64
+// conversions and scaling (Eq. A4, with a division per bin: 1.81), 0.846 (0.902)
+// with these.  Two pairs per thread: the kernel alone takes 405 us there, with
+// 1, 4 or 16 pairs 440, 546 and 535 (256 FP64 curves of 2^16: 179, 184, 178 and
+// 184).
+constexpr uint32_t kPgPairs = 512;
 
 // (x^2 + y^2) 2^-sh, rounded once: a float's square is exact in FP64.
 __device__ __forceinline__ double power_of(float x, float y, int sh)
@@ -62,14 +64,19 @@ __global__ void __launch_bounds__(256) k_periodogram(const int* __restrict__ cls
     const uint32_t k0 = blockIdx.x % chunks * pairs;
     const V* __restrict__ Z = (const V*)Zin + (cv.off >> 1);
     double* __restrict__ out = P + cv.offh;
-    // 2 / N^2 = 2^-sh, or the rms normalisation
+    // 2 / N^2 = 2^-sh, or the rms normalisation (by one thread: its division is
+    // as many FP64 operations as a pair's bins)
     const int sh = rms ? 0 : 2 * (int)log2M + 1;
-    double scale = 1.0;
+    __shared__ double rms_scale;
     if (rms) {
-        const V z0 = Z[0];
-        const double X0 = (double)(z0.x + z0.y);
-        scale = 2.0 * cv.dt * nd / (X0 * X0);
+        if (threadIdx.x == 0) {
+            const V z0 = Z[0];
+            const double X0 = (double)(z0.x + z0.y);
+            rms_scale = 2.0 * cv.dt * nd / (X0 * X0);
+        }
+        __syncthreads();
     }
+    const double scale = rms ? rms_scale : 1.0;
     auto power = [&](T x, T y) -> double {
         const double v = power_of(x, y, sh);
         return rms ? v * scale : v;
@@ -282,9 +289,9 @@ static void launch_structure(const Plan& p, const ClassInfo& k, int nlags, const
             k.d_curves, p.d_curves, k.ncurves, k.log2n, segs, nlags, p.d_lags, part, out);
 }
 
-// kPgPairs pairs per block where that gives two blocks per SM, fewer (down to
-// one per thread) where not: with their transform, one 2^16 FP32 curve
-// 18 us (kPgPairs per block: 29), 64 of 2^14 26 (35), one 2^16 FP64 curve 32 (56).
+// kPgPairs pairs per block where that gives two blocks per SM, one per thread
+// where not: with their transform, one 2^16 FP32 curve 19 us (4096 pairs per
+// block: 29), 64 of 2^14 24 (35), one 2^16 FP64 curve 32 (56).
 template <typename T>
 static void launch_periodogram(const Plan& p, const ClassInfo& k, const void* Z, int rms, double* out, cudaStream_t st)
 {
