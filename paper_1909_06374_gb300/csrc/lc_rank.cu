@@ -41,28 +41,6 @@ struct RankCta {
     static_assert(BYTES <= 227 * 1024 && R::NSEG + 1 <= kRankBounds, "one CTA's shared memory");
 };
 
-// Bitonic sort of (key, pos) pairs held in two shared arrays.
-template <int TH, typename K>
-__device__ __forceinline__ void cta_bitonic_pairs(K* key, uint16_t* pos, int n)
-{
-    for (int k = 2; k <= n; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < n / 2; i += TH) {
-                const int e = ((i & ~(j - 1)) << 1) | (i & (j - 1));
-                const K a = key[e], b = key[e + j];
-                const uint16_t pa = pos[e], pb = pos[e + j];
-                if ((b < a || (b == a && pb < pa)) == ((e & k) == 0)) {
-                    key[e] = b;
-                    key[e + j] = a;
-                    pos[e] = pb;
-                    pos[e + j] = pa;
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
 // VALUES: out = the sorted values; else out[position] = s_in[rank].  out may be
 // src: every value is in shared memory before the first barrier.
 template <typename T, int LOG2L, bool VALUES>
@@ -109,19 +87,24 @@ __global__ void __launch_bounds__(RankCta<T, LOG2L>::TH) k_rank_cta(const RankAr
         if (bounds && tid <= C::R::NSEG) bounds[tid] = m.spl[tid];
     } else {  // crowded bins (many equal values): sorted whole
         __syncthreads();
+        K v[PER];
 #pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            key[tid + j * TH] = rank_key(val(j));  // each thread its own values
-            m.slot[tid + j * TH] = (uint16_t)(tid + j * TH);
-        }
+        for (int j = 0; j < PER; ++j) v[j] = rank_key(val(j));
         __syncthreads();
-        cta_bitonic_pairs<TH>(key, m.slot, L);
-        const T* __restrict__ s = (const T*)a.s_in + off;
+        const SortPairs<K> sp{key, m.slot};
 #pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const int i = tid + j * TH;
-            if (VALUES) out[i] = key_value(key[i]);
-            else out[m.slot[i]] = s[i];
+        for (int j = 0; j < PER; ++j) sp.store(tid + j * TH, {v[j], (uint32_t)(tid + j * TH)});
+        __syncthreads();
+        if constexpr (VALUES) {
+            const SortValues<K> sv{key};
+            cta_bitonic<TH>(sv, L);
+#pragma unroll
+            for (int j = 0; j < PER; ++j) out[tid + j * TH] = key_value(sv.load(tid + j * TH));
+        } else {
+            cta_bitonic<TH>(sp, L);
+            const T* __restrict__ s = (const T*)a.s_in + off;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) out[sp.load(tid + j * TH).p] = s[tid + j * TH];
         }
         if (bounds && tid <= C::R::NSEG) bounds[tid] = 0.0f;  // the next iteration finds them useless
     }

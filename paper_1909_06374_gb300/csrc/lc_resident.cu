@@ -340,7 +340,7 @@ struct CtaShape {
 };
 
 // x[position] = s[rank] of the L values in xf (swizzled); idle: the other
-// transform buffer; both: the two of them.  Ends with a block barrier.
+// transform buffer.  Ends with a block barrier.
 template <int LOG2L>
 __device__ __forceinline__ void rank_replace(float* xf, float2* idle, unsigned char* smem, const float* s,
                                              uint32_t* wsum, bool& warm)
@@ -366,15 +366,15 @@ __device__ __forceinline__ void rank_replace(float* xf, float2* idle, unsigned c
 #pragma unroll
         for (int j = 0; j < PER; ++j) xf[fsw(tid + j * TH)] = s[rk[j]];
     } else {  // crowded: sorted whole, by (order key, position)
-        unsigned long long* both = (unsigned long long*)smem;
+        const SortValues<unsigned long long> both{(unsigned long long*)smem};
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < PER; ++j)
-            both[tid + j * TH] = ((unsigned long long)order_key(v[j]) << 32) | (uint32_t)(tid + j * TH);
+            both.store(tid + j * TH, ((unsigned long long)order_key(v[j]) << 32) | (uint32_t)(tid + j * TH));
         __syncthreads();
         cta_bitonic<TH>(both, CS::L);
 #pragma unroll
-        for (int j = 0; j < PER; ++j) rk[j] = (uint32_t)both[tid + j * TH];
+        for (int j = 0; j < PER; ++j) rk[j] = (uint32_t)both.load(tid + j * TH);
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < PER; ++j) xf[fsw((int)rk[j])] = s[tid + j * TH];

@@ -38,6 +38,19 @@ def test_every_state_gives_a_permutation_of_the_draws(prec, log2ns, monkeypatch)
                 assert np.array_equal(np.sort(got[seg]), s[seg]), (l, name, iters)
 
 
+@pytest.mark.parametrize("prec,log2ns", [(LC_FP32, [10, 11, 12, 14]), (LC_FP64, [10, 11, 12, 13, 14])])
+def test_sorted_draws_of_a_narrow_range(prec, log2ns):
+    """Draws that are equal in float, so that every bin is crowded: sorted whole."""
+    jobs = [workloads.job(l, 1, seed=60 + c, curve_id=c, log_lmin=-1.0, log_lmax=-1.0 + 1e-9, log_lbreak=-1.0 + 5e-10)
+            for c, l in enumerate(log2ns)]
+    with Plan(jobs, prec) as p:
+        p.setup()
+        x, s = p.get_state().cpu().numpy(), p.buffer(2).cpu().numpy()
+        for c in range(len(jobs)):
+            seg = slice(p.offsets[c], p.offsets[c + 1])
+            assert np.array_equal(np.sort(x[seg]), s[seg])
+
+
 @pytest.mark.parametrize("prec", [LC_FP32, LC_FP64])
 @pytest.mark.parametrize("iters", [7, 8, 11, 32, 101])
 def test_graphs_with_a_remainder(prec, iters):
