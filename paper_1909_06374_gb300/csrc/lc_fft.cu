@@ -214,8 +214,8 @@ constexpr int kSmallThreads = 128;
 // The radix-QA sub-pass of span 2^log2p2 on the tile and the radix-QB one after
 // it, in registers between the two: a butterfly of the second takes one output
 // of each of QB first ones, R/(QA QB) apart.  QA = 1: the second one alone.
-// FIRST (of span 1): the first has no twiddles, and the second's, powers of
-// W_{QA QB}, are taken without the multiplications by 1 and -+i.
+// FIRST, of a pair of span 1: the first has no twiddles, and the second's, powers
+// of W_{QA QB}, are taken without the multiplications by 1 and -+i.
 template <typename T, int QA, int QB, bool FIRST, bool INV, int LR, int C, int TH>
 __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2p2, const cplx<T>* __restrict__ tR)
 {
@@ -276,7 +276,7 @@ __device__ __forceinline__ void tile_subpass(cplx<T>* __restrict__ buf, int log2
                     for (int m = 0; m < QB; ++m) u[bi][m * QA + q] = w[q][m];
                 }
             } else {
-                if (!FIRST) {
+                if (p2 > 1) {
 #pragma unroll
                     for (int q = 1; q < QB; ++q) u[bi][q] = turn(u[bi][q], (q * k2) << (LR - LB - log2p2));
                 }
@@ -303,20 +303,20 @@ template <typename T, bool INV, int LR, int C, int TH>
 __device__ __forceinline__ void tile_dft(cplx<T>* __restrict__ buf, const cplx<T>* __restrict__ tR)
 {
     constexpr int LQ = sizeof(T) == 8 ? 2 : 4;
-    constexpr int L0 = LR % LQ ? LR % LQ : LQ;  // the first sub-pass
+    constexpr int rem = LR % LQ;
     constexpr bool PAIRS = sizeof(T) == 8 && C > kSmallCols && LR >= 7;
     int log2p2 = 0;
     if constexpr (PAIRS) {
-        tile_subpass<T, (1 << L0), 4, true, INV, LR, C, TH>(buf, 0, tR);
-        log2p2 = L0 + 2;
+        tile_subpass<T, (rem ? 2 : 4), 4, true, INV, LR, C, TH>(buf, 0, tR);
+        log2p2 = rem ? 3 : 4;
         __syncthreads();
         for (; log2p2 + 4 <= LR; log2p2 += 4) {
             tile_subpass<T, 4, 4, false, INV, LR, C, TH>(buf, log2p2, tR);
             __syncthreads();
         }
-    } else {
-        tile_subpass<T, 1, (1 << L0), true, INV, LR, C, TH>(buf, 0, tR);
-        log2p2 = L0;
+    } else if constexpr (rem != 0) {
+        tile_subpass<T, 1, (1 << rem), false, INV, LR, C, TH>(buf, 0, tR);
+        log2p2 = rem;
         __syncthreads();
     }
     for (; log2p2 < LR; log2p2 += LQ) {
