@@ -66,6 +66,24 @@ SORT_PLACE_LOG2 = 26         # lengths from here on store the argsort's result b
 FUSED_LOG2 = (10, 14)        # FP32 lengths the one-CTA fused kernel can take
 
 
+def fused_curve_ids(jobs, esize, fused_elements):
+    """ids of the jobs that the fused kernels run: those of 2^10..2^top for the
+    top length whose samples add up to the plan's fused samples; None without
+    such a top."""
+    for top in range(FUSED_LOG2[0] - 1, FUSED_LOG2[1] + 1):
+        fused_len = [j for j in jobs if esize == 4 and FUSED_LOG2[0] <= int(j["log2n"]) <= top]
+        if sum(1 << int(j["log2n"]) for j in fused_len) == fused_elements:
+            return {id(j) for j in fused_len}
+    return None
+
+
+def rank_cta_elements(jobs, esize, fused_elements):
+    """Samples of the multi-kernel curves that one CTA per curve ranks."""
+    lo, hi = RANK_CTA_LOG2[esize]
+    fused = fused_curve_ids(jobs, esize, fused_elements) or set()
+    return sum(1 << int(j["log2n"]) for j in jobs if lo <= int(j["log2n"]) <= hi and id(j) not in fused)
+
+
 def scheduled_bytes_per_sample_iter(jobs, esize, fused_elements, radix_only=True):
     """HBM bytes the scheduled kernels move per sample-iteration (reads +
     writes at their algorithmic sizes), averaged over the batch's
@@ -80,17 +98,11 @@ def scheduled_bytes_per_sample_iter(jobs, esize, fused_elements, radix_only=True
     three values per element where one CTA ranks a curve whole, and the
     position buckets of the longest radix-sorted curves (16 and 24 B).  Fused curves touch
     HBM once per launch of all iterations: 14 B per sample (FP32) / iterations.
-    The fused curves are those of 2^10..2^top for the top length whose
-    samples add up to the plan's fused samples (the path table's crossover,
-    2^12 built in, or LC_RESIDENT_MAX_LOG2); with no such top the figure is
-    not defined (None).  Without the Eq. 4 pass."""
+    The fused curves are fused_curve_ids' (the path table's crossover, 2^12
+    built in, or LC_RESIDENT_MAX_LOG2); without them the figure is not defined
+    (None).  Without the Eq. 4 pass."""
     fp32 = esize == 4
-    fused_ids = None
-    for top in range(FUSED_LOG2[0] - 1, FUSED_LOG2[1] + 1):
-        fused_len = [j for j in jobs if fp32 and FUSED_LOG2[0] <= int(j["log2n"]) <= top]
-        if sum(1 << int(j["log2n"]) for j in fused_len) == fused_elements:
-            fused_ids = {id(j) for j in fused_len}
-            break
+    fused_ids = fused_curve_ids(jobs, esize, fused_elements)
     if fused_ids is None:
         return None
     tot_b, tot_si = 0.0, 0
@@ -455,8 +467,7 @@ def gpu_line(args, workload, steps, warmup, dist, e2e_on, cpu_on, extra=False):
             dominant = "sort_scatter"
             launches_k = max(1, prof["scatter_launches"])
             nb = prof.get("bucket_elements", 0)
-            lo, hi = RANK_CTA_LOG2[esize]
-            nc = sum(1 << int(j["log2n"]) for j in jobs if lo <= int(j["log2n"]) <= hi) if not prof["fused_elements"] else 0
+            nc = rank_cta_elements(jobs, esize, prof["fused_elements"])
             nr = prof["sorted_elements"] - nb - nc
             # every element of a radix-sorted class goes through all passes; every
             # element of a sample-sorted class through the bucket scatter and finish
