@@ -4,13 +4,20 @@
 // bits.  The FP64 logarithm, quotients and exponential behind it are ~120
 // double operations, and this GPU runs 2 of them per clock and SM against 128
 // float ones.  Here the argument of the logarithm (or the table's u) is formed
-// with the same FP64 operations as before (5 to 9 of them), and log2(lambda)
+// with the FP64 sequence's own operations (5 to 9 of them), and log2(lambda)
 // and lambda are then carried in pairs of floats (head + tail, error-free
 // sums and products after Dekker 1971 and Knuth, TAOCP 4.2.2; table-driven
-// reductions after Tang, ACM TOMS 1989/1990) to about 2^-39.  Where every
-// value within the error bound rounds to the same float, that float is the
-// draw; otherwise (about 1 draw in 2^11) the caller runs the FP64 sequence.
-// So the draws keep their bits.
+// reductions after Tang, ACM TOMS 1989/1990).  With log2(lambda) = E = B + L K,
+// relative errors of lambda (times ln 2 where they are E's):
+//   2^-39  the float polynomial of 2^g: its terms reach 2^-16, rounded to
+//          2^-40 a few times, and the first one left out is 2^-44;
+//   (|E| + kc) 2^-44  B, K, the pair product L K and L itself, each to 2^-46 of
+//          its share (log_pair: 2^-45 + 2^-47 |L|, times K).
+// exp2_pair allows four times that, 2^-37 + (|E| + kc) 2^-42, beside which the
+// FP64 sequence's own rounding (2^-50) does not count.  Where every value
+// within that bound rounds to the same float, that float is the draw; otherwise
+// (about 1 draw in 2^11) the caller runs the FP64 sequence.  So the draws keep
+// their bits.  FP64 pipe 86% busy (512 curves of 2^16).
 #pragma once
 #include "lc_common.cuh"
 

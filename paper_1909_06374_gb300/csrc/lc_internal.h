@@ -252,10 +252,13 @@ template <typename T> void launch_fft_iteration(const Plan& p, const std::vector
 template <typename T> void launch_spectral_tk(const Plan& p, const ClassInfo& k, void* Zp, cudaStream_t st);
 
 // sort stage (lc_sort.cu)
-// shortest length whose argsort stores its result by position buckets (the
-// state, 256 MB in FP32, no longer fits the 129 MB L2; 2^28 samples, ms per
-// iteration direct / by buckets: 2^24 11.7 / 12.2, 2^25 12.6 / 12.5, 2^26
-// 14.3 / 12.9)
+// shortest length whose argsort stores its result by position buckets, in both
+// precisions (2^28 FP32 samples, ms per iteration direct / by buckets: 2^24 11.7
+// / 12.2, 2^25 12.6 / 12.5, 2^26 14.3 / 12.9, where the 256 MB of a state no
+// longer fit the 129 MB L2; two FP64 curves of 2^25, 256 MB as well, but fewer
+// and wider scattered stores, scatters 4.61 / 4.73).  It pays for scattered
+// positions: one curve of 2^26 equal or presorted values takes 2.0 ms to rank,
+// 1.6 with direct stores (normal ones 2.65 against 4.1).
 constexpr uint32_t kSortPlaceMinLog2 = 26;
 constexpr int kSortTile = 2048;
 constexpr int kScanChunk = 32;

@@ -21,7 +21,7 @@ namespace lc {
 //
 // One block takes `pairs` conjugate pairs of one curve (launch_periodogram).  A
 // float bin's power takes two FP64 operations (three for Eq. A4) of the 2 per
-// clock and SM: its conversions and Eq. A2's scale, a power of two, are put
+// clock and SM, whose pipe is the limit (86% busy): its conversions and Eq. A2's scale, a power of two, are put
 // together from bits.  2048 curves of 2^16 samples, transform included: 1.11 ms with FP64
 // conversions and scaling (Eq. A4, with a division per bin: 1.81), 0.846 (0.902)
 // with these.  Two pairs per thread: the kernel alone takes 405 us there, with
@@ -50,9 +50,9 @@ __device__ __forceinline__ double power_of(double x, double y, int sh)
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_periodogram(const int* __restrict__ cls_curves,
-                                                     const CurveDev* __restrict__ curves, uint32_t pairs, uint32_t log2M,
-                                                     const void* __restrict__ tw, const void* __restrict__ Zin, int rms,
-                                                     double* __restrict__ P)
+                                                     const CurveDev* __restrict__ curves, uint32_t pairs,
+                                                     uint32_t log2M, const void* __restrict__ tw,
+                                                     const void* __restrict__ Zin, int rms, double* __restrict__ P)
 {
     using V = cplx<T>;
     const uint32_t half = 1u << (log2M - 1);
@@ -112,8 +112,9 @@ __global__ void __launch_bounds__(256) k_periodogram(const int* __restrict__ cls
 // costs one load (of x_{i+tau}, mostly from L1: neighbouring lags read
 // overlapping windows), a subtraction and a multiply-add, all of a run's loads
 // independent.  256 curves of 2^16 samples at 53 lags: 0.23 ms (3.8e12
-// pairs/s), bound by the loads' L1 and L2 traffic; one block per (curve, lag)
-// that walks the whole curve, two loads per pair and nothing kept: 3.14 ms.
+// pairs/s), bound by the loads through L1 (68% of its throughput, 96% of them
+// hits; issue 57%); one block per (curve, lag) that walks the whole curve, two
+// loads per pair and nothing kept: 3.14 ms.
 constexpr int kSfBatch = 16;  // lags whose runs are added up together
 
 // Sum of the 256 runs at r (>= 0, or NaN) by a warp, in lane 0.  Added as

@@ -5,7 +5,8 @@
 // the positions of shared bins' members, counters and starts take 208 KB at 2^14);
 // FP32 ones of 2^10 .. 2^12, whose iterations the fused kernels run, for their
 // draws and on the multi-kernel path (2^13 on: the sample sort).
-// Bound by issue and shared-memory latency on the one SM of a curve.  One FP64
+// Bound by latency on the one SM of a curve (512 FP64 curves of 2^14: issue 34%,
+// ALU 38%, stalls on global loads first, one CTA of 32 warps per SM).  One FP64
 // curve of 2^14 samples, transforms included: 119 us per iteration with eight
 // LSD passes (24 launches), 94 with FP64 conversions and comparisons here, 72
 // with integer ones.
@@ -114,7 +115,8 @@ template <typename T, int LOG2L>
 cudaError_t rank_attr()
 {
     const int smem = (int)RankCta<T, LOG2L>::BYTES;
-    cudaError_t e = cudaFuncSetAttribute(k_rank_cta<T, LOG2L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e =
+        cudaFuncSetAttribute(k_rank_cta<T, LOG2L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_rank_cta<T, LOG2L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return e;

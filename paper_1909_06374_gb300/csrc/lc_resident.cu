@@ -734,8 +734,9 @@ cudaError_t resident_kernel_attributes()
 // fused vs multi-kernel: 2^10 4.8e10 vs 4.1e10, 2^11 7.1e10 vs 4.9e10, 2^12
 // 8.7e10 vs 4.5e10, 2^13 6.9e10 vs 4.4e10, 2^14 4.5e10 vs 4.7e10, 2^15 2.2e10
 // for the 2-CTA cluster kernel vs 4.9e10).  The two paths' transforms round
-// differently, so 2^13 stays where its results have been.  LC_RESIDENT_MAX_LOG2 (up to 14 for the one-CTA kernel) moves it;
-// LC_PATH=resident also runs the cluster kernels at 2^15 and 2^16.
+// differently, so 2^13 stays where its results have been.  LC_RESIDENT_MAX_LOG2
+// (up to 14 for the one-CTA kernel) moves it; LC_PATH=resident also runs the
+// cluster kernels at 2^15 and 2^16.
 bool resident_supported(const Plan& p, uint32_t log2n)
 {
     if (p.prec != LC_FP32 || log2n < kResMinLog2) return false;
