@@ -39,13 +39,16 @@ struct RankCta {
     static constexpr size_t SEG = SLOT + R::SLOT;
     static constexpr size_t SPL = SEG + R::SEG;
     static constexpr size_t BYTES = SPL + R::SPL;
+    // resident CTAs per SM that the ranking's registers allow; the crowded
+    // curves' sort, which takes more, gives way
+    static constexpr int MINB = LOG2L <= 11 ? 3 : LOG2L == 12 ? 2 : 1;
     static_assert(BYTES <= 227 * 1024 && R::NSEG + 1 <= kRankBounds, "one CTA's shared memory");
 };
 
 // VALUES: out = the sorted values; else out[position] = s_in[rank].  out may be
 // src: every value is in shared memory before the first barrier.
 template <typename T, int LOG2L, bool VALUES>
-__global__ void __launch_bounds__(RankCta<T, LOG2L>::TH) k_rank_cta(const RankArgs a)
+__global__ void __launch_bounds__(RankCta<T, LOG2L>::TH, RankCta<T, LOG2L>::MINB) k_rank_cta(const RankArgs a)
 {
     using C = RankCta<T, LOG2L>;
     using K = typename key_of<T>::type;
