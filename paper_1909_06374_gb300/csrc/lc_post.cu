@@ -121,8 +121,8 @@ constexpr int kSfBatch = 16;  // lags whose runs are added up together
 // integers, 2^-54 of the largest run's power of two as unit: exact for the runs
 // above 2^-31 of it, and below 2^-46 of the sum in all (255 FP64 additions:
 // 2^-45), over the whole range of float.  256 curves of 2^16 samples at 53 lags
-// 233 us, with FP64 additions (16 clocks per warp operation) 258; 2000 curves of
-// 2^10 at 27 lags 62 against 117.  Infinities and NaN go there.
+// 232 us, with FP64 additions (16 clocks per warp operation) 258; 2000 curves of
+// 2^10 at 27 lags 61 against 117.  Infinities and NaN go there.
 __device__ __forceinline__ double sum_runs(const float* r)
 {
     const int lane = threadIdx.x & 31;
@@ -146,8 +146,11 @@ __device__ __forceinline__ double sum_runs(const float* r)
         const uint32_t m = e ? (v & 0x7fffffu) | 0x800000u : v;
         acc += ((unsigned long long)m << 31) >> min(et - max(e, 1u), 63u);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    // the lanes' 58 bits in three parts whose sums fit a word
+    const uint32_t p0 = __reduce_add_sync(0xffffffffu, (uint32_t)acc & 0x7ffffffu);
+    const uint32_t p1 = __reduce_add_sync(0xffffffffu, (uint32_t)(acc >> 27) & 0x7ffffffu);
+    const uint32_t p2 = __reduce_add_sync(0xffffffffu, (uint32_t)(acc >> 54));
+    acc = p0 + ((unsigned long long)p1 << 27) + ((unsigned long long)p2 << 54);
     return (double)acc * __hiloint2double((int)((1023u + et - 181u) << 20), 0);
 }
 
