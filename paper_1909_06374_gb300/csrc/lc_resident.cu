@@ -339,6 +339,13 @@ struct CtaShape {
     static constexpr int MINB = LOG2L <= 12 ? 2 : 1;
 };
 
+// Sort of a crowded curve, out of line: inside the iteration it costs registers
+// (50 iterations of 8000 curves of 2^10 7.77 -> 7.90 ms).
+__device__ __noinline__ void sort_crowded(unsigned long long* v, int n)
+{
+    cta_bitonic<kResThreads>(SortValues<unsigned long long>{v}, n);
+}
+
 // x[position] = s[rank] of the L values in xf (swizzled); idle: the other
 // transform buffer.  Ends with a block barrier.
 template <int LOG2L>
@@ -372,7 +379,7 @@ __device__ __forceinline__ void rank_replace(float* xf, float2* idle, unsigned c
         for (int j = 0; j < PER; ++j)
             both.store(tid + j * TH, ((unsigned long long)order_key(v[j]) << 32) | (uint32_t)(tid + j * TH));
         __syncthreads();
-        cta_bitonic<TH>(both, CS::L);
+        sort_crowded(both.v, CS::L);
 #pragma unroll
         for (int j = 0; j < PER; ++j) rk[j] = (uint32_t)both.load(tid + j * TH);
         __syncthreads();
